@@ -46,7 +46,10 @@ __global__ void __launch_bounds__(kAdjBlock) adj_prepare_kernel(int64_t nvox, co
                                                                 double* __restrict__ Ct21, double* __restrict__ a_u,
                                                                 double* __restrict__ yK) {
   const double gs[6] = {gs0, gs1, gs2, gs3, gs4, gs5};
-  const Step hs = make_step(h);
+  __shared__ RayConst ray[kMaxPhases];
+  if (threadIdx.x < kMaxPhases && tab->kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV)
+    ray[threadIdx.x] = make_ray(tab->p64[threadIdx.x], h);
+  __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nvox; base += stride) {
     const int64_t i = base + threadIdx.x;
@@ -59,9 +62,8 @@ __global__ void __launch_bounds__(kAdjBlock) adj_prepare_kernel(int64_t nvox, co
       e[c] = in ? eps_k[c * nvox + i] : 0.0;
       zi[c] = vp ? zprev[c * nvox + i] : 0.0;
     }
-    if constexpr (MODE == MODE_FP64) voxel_fp64<NortonDev>(tab->p64[ph], e, zi, hs, vp, s, zo, nullptr);
-    else voxel_fp32_fix<NortonDev>(tab->p64[ph], tab->p32[ph], e, zi, hs, vp, s, zo, nullptr);
     if (!in) continue;
+    if (vp) voxel_ray<NortonDev>(ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<double*>(nullptr));
     double C[6][6], au[6];
     if (vp) {
       const LawParams<double>& p = tab->p64[ph];

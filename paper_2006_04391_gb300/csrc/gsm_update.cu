@@ -26,17 +26,9 @@ constexpr int kBlock = 128;
 
 template <class T> __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 
-// Viscoplastic (Norton) voxels.  The FP32-bulk update without tangent is
-// held to kFixBlocks blocks of 128 threads per SM (128 registers at 4): its
-// FP64 and double-float correction needs the warps to hide the FP64 pipe's
-// latency.
-#ifndef GSM_FIX_BLOCKS
-#define GSM_FIX_BLOCKS 4
-#endif
-constexpr int kFixBlocks = GSM_FIX_BLOCKS;
+// Viscoplastic (Norton) voxels.
 template <int MODE, bool TAN>
-__global__ void __launch_bounds__(kBlock, (MODE == MODE_FP32_FIX && !TAN) ? kFixBlocks : 1) norton_kernel(int64_t n, int64_t ld, LawParams<double> p,
-                                                        LawParams<float> pf, Step hs,
+__global__ void __launch_bounds__(kBlock) norton_kernel(int64_t n, int64_t ld, const __grid_constant__ RayConst rc,
                                                         const void* __restrict__ eps_,
                                                         const void* __restrict__ zn_, void* __restrict__ sig_,
                                                         void* __restrict__ z_, void* __restrict__ tan_,
@@ -48,7 +40,6 @@ __global__ void __launch_bounds__(kBlock, (MODE == MODE_FP32_FIX && !TAN) ? kFix
   IO* z = static_cast<IO*>(z_);
   IO* tan = static_cast<IO*>(tan_);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const NortonDf cdf = norton_df(p, hs.inv_h);  // formed once per thread (FP32_FIX)
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
     const int64_t i = base + threadIdx.x;
     const bool active = i < n;
@@ -59,14 +50,7 @@ __global__ void __launch_bounds__(kBlock, (MODE == MODE_FP32_FIX && !TAN) ? kFix
       zi[c] = active ? ldg(zn + c * ld + i) : IO(0);
     }
     IO t[21];
-    unsigned st;
-    if constexpr (MODE == MODE_FP64) {
-      st = voxel_fp64<NortonDev>(p, e, zi, hs, active, s, zo, TAN ? t : nullptr);
-    } else if constexpr (MODE == MODE_FP32_FIX) {
-      st = voxel_fp32_fix<NortonDev>(p, pf, e, zi, hs, active, s, zo, TAN ? t : nullptr, nullptr, &cdf);
-    } else {
-      st = voxel_fp32<NortonDev>(pf, e, zi, hs, active, s, zo, TAN ? t : nullptr);
-    }
+    unsigned st = voxel_ray<NortonDev>(rc, e, zi, active, MODE == MODE_FP32_FIX, s, zo, TAN ? t : nullptr);
     bool fin = true;
 #pragma unroll
     for (int c = 0; c < 6; ++c) fin = fin && finite64(s[c]) && finite64(zo[c]);
@@ -132,7 +116,7 @@ template <auto Kernel> int grid_for(int64_t n) {
 template <int MODE, bool TAN>
 cudaError_t launch_norton(const Material& m, int64_t n, int64_t ld, double h, const void* eps, const void* zn,
                           void* sig, void* z, void* tan, int32_t* status, cudaStream_t s) {
-  norton_kernel<MODE, TAN><<<grid_for<norton_kernel<MODE, TAN>>(n), kBlock, 0, s>>>(n, ld, m.p64, m.p32, make_step(h), eps, zn, sig, z, tan, status);
+  norton_kernel<MODE, TAN><<<grid_for<norton_kernel<MODE, TAN>>(n), kBlock, 0, s>>>(n, ld, make_ray(m.p64, h), eps, zn, sig, z, tan, status);
   count_launch();
   return cudaGetLastError();
 }

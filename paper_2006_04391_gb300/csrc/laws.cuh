@@ -56,6 +56,9 @@ struct Elastic {
 // c_phi = sigma0 edot0 n/(n+1) edot0^(-(n+1)/n).
 struct NortonDev {
   static constexpr int NY = 5;
+  // psi and phi measure the same deviatoric norm: the implicit-Euler step is a
+  // scalar equation on the predictor ray (ray.cuh)
+  static constexpr bool kRay = true;
 
   template <class EP, class YP, class P> AD_HD static auto psi(const EP& e, const YP& y, const P& p) {
     using ad::get;

@@ -52,6 +52,7 @@ struct Reduced {
 
 // One job of a batched launch (device copy, rebuilt by the host every tick).
 struct JobView {
+  RayConst ray[kMaxPhases];  // the scalar equation of each Norton phase at this step's h
   const uint8_t* phase;
   const void* eps_raw;   // [6][nvox] N^3 * strain (C2R output)
   const void* zn;        // [6][nvox]
@@ -66,7 +67,7 @@ struct JobView {
   int64_t vchunk0, mchunk0;  // first chunk of this job in its launch
   int n_vch, n_mch;
   int N;
-  int warm;              // 1: z holds this job's previous evaluation of the current step (warm start)
+  int pad1;
   double h, inv_h, inv_n3, lam0, mu0;
   // ode23 laws (Sec. 4.3): strain at t_n, the Michel-Suquet alpha, tolerances
   const double* eps_prev;  // [6][nvox]
@@ -109,49 +110,32 @@ template <int NV> __device__ void block_sum(double (&v)[NV], double* out, int64_
   block_sum_at<NV>(v, out, stride, blockIdx.x);
 }
 
-// Material evaluation of voxel i.  Every lane of a warp must call this (the
-// Newton loops vote warp-wide); lanes with in = false only vote.  The field
-// precision T is also that of the 1/N^3 scaling and of the lane's partial
-// stress sums (FP32 fields: no FP64 work, a sixty-fourth of the FP32 rate on
-// GB300, outside the law; the block sums are FP64).
+// Material evaluation of voxel i.  The field precision T is also that of the
+// 1/N^3 scaling and of the lane's partial stress sums (FP32 fields: no FP64
+// work, a sixty-fourth of the FP32 rate on GB300; the block sums are FP64).
 template <class T, int MODE>
-__device__ __forceinline__ void material_voxel(int64_t i, bool in, int64_t nvox, const uint8_t* __restrict__ phase,
-                                               const PhaseTable& tab, const Step& hs, T inv_n3,
+__device__ __forceinline__ void material_voxel(int64_t i, int64_t nvox, const uint8_t* __restrict__ phase,
+                                               const PhaseTable& tab, const RayConst* ray, T inv_n3,
                                                const T* __restrict__ eps_raw, const T* __restrict__ zn,
-                                               T* __restrict__ sig, T* __restrict__ z, T (&acc)[6],
-                                               bool warm = false) {
-  const int ph = in ? (int)phase[i] : 0;
-  const bool vp = in && tab.kind[ph] == GSM_PSI_ELASTIC_VP_DEV;
-  T e[6], zi[6], s[6], zo[6], zp[6];
+                                               T* __restrict__ sig, T* __restrict__ z, T (&acc)[6]) {
+  const int ph = (int)phase[i];
+  T e[6], s[6], zo[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    e[c] = in ? __ldg(eps_raw + c * nvox + i) * inv_n3 : T(0);
-    zi[c] = vp ? __ldg(zn + c * nvox + i) : T(0);
-    // warm start: this voxel's z from the previous evaluation of the step
-    // (read before this evaluation overwrites it)
-    zp[c] = (warm && vp) ? z[c * nvox + i] : zi[c];
-  }
-  const T* zprev = warm ? zp : nullptr;
-  if constexpr (MODE == MODE_FP64) {
-    voxel_fp64<NortonDev>(tab.p64[ph], e, zi, hs, vp, s, zo, nullptr, zprev);
-  } else if constexpr (MODE == MODE_FP32_FIX) {
-    voxel_fp32_fix<NortonDev>(tab.p64[ph], tab.p32[ph], e, zi, hs, vp, s, zo, nullptr, zprev);
+  for (int c = 0; c < 6; ++c) e[c] = __ldg(eps_raw + c * nvox + i) * inv_n3;
+  if (tab.kind[ph] == GSM_PSI_ELASTIC_VP_DEV) {
+    T zi[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) zi[c] = __ldg(zn + c * nvox + i);
+    voxel_ray<NortonDev>(ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<T*>(nullptr));
   } else {
-    voxel_fp32<NortonDev>(tab.p32[ph], e, zi, hs, vp, s, zo, nullptr, zprev);
-  }
-  if (in && !vp) {
     if constexpr (sizeof(T) == 8) voxel_elastic<double>(tab.p64[ph], e, s, nullptr);
     else voxel_elastic<float>(tab.p32[ph], e, s, nullptr);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) zo[c] = T(0);
   }
-  if (in) {
 #pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      sig[c * nvox + i] = s[c];
-      z[c * nvox + i] = zo[c];
-      acc[c] += s[c];
-    }
+  for (int c = 0; c < 6; ++c) {
+    sig[c * nvox + i] = s[c];
+    z[c * nvox + i] = zo[c];
+    acc[c] += s[c];
   }
 }
 
@@ -309,16 +293,18 @@ __device__ __forceinline__ void gamma_pair_f32(int N, float inv2mu, float coef, 
 // sum per block).  Used by the allocation-free entry point.
 template <class T, int MODE>
 __global__ void __launch_bounds__(kMatBlock) ms_material_kernel(int64_t nvox, const uint8_t* __restrict__ phase,
-                                                                PhaseTable tab, Step hs, double inv_n3,
+                                                                PhaseTable tab, double h, double inv_n3,
                                                                 const T* __restrict__ eps_raw,
                                                                 const T* __restrict__ zn, T* __restrict__ sig,
                                                                 T* __restrict__ z, double* __restrict__ partials) {
+  __shared__ RayConst ray[kMaxPhases];
+  if (threadIdx.x < kMaxPhases && tab.kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV)
+    ray[threadIdx.x] = make_ray(tab.p64[threadIdx.x], h);
+  __syncthreads();
   T acc[6] = {0, 0, 0, 0, 0, 0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nvox; base += stride) {
-    const int64_t i = base + threadIdx.x;
-    material_voxel<T, MODE>(i, i < nvox, nvox, phase, tab, hs, (T)inv_n3, eps_raw, zn, sig, z, acc);
-  }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += stride)
+    material_voxel<T, MODE>(i, nvox, phase, tab, ray, (T)inv_n3, eps_raw, zn, sig, z, acc);
   double accd[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) accd[c] = (double)acc[c];
@@ -345,14 +331,13 @@ __global__ void __launch_bounds__(kMatBlock) ms_material_batch_kernel(const JobV
   for (int64_t gc = blockIdx.x; gc < total_chunks; gc += gridDim.x) {
     const JobView& v = views[owner(starts, n_jobs, gc)];
     const int64_t lc = gc - v.vchunk0;
-    const Step hs{v.h, v.inv_h, (float)v.h, (float)v.inv_h};
     T acc[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 1
     for (int sweep = 0; sweep < kVChunk / kMatBlock; ++sweep) {
       const int64_t i = lc * kVChunk + sweep * kMatBlock + threadIdx.x;
-      material_voxel<T, MODE>(i, i < v.nvox, v.nvox, v.phase, *v.tab, hs, (T)v.inv_n3,
-                              static_cast<const T*>(v.eps_raw), static_cast<const T*>(v.zn),
-                              static_cast<T*>(v.sig), static_cast<T*>(v.z), acc, v.warm != 0);
+      if (i < v.nvox)
+        material_voxel<T, MODE>(i, v.nvox, v.phase, *v.tab, v.ray, (T)v.inv_n3, static_cast<const T*>(v.eps_raw),
+                                static_cast<const T*>(v.zn), static_cast<T*>(v.sig), static_cast<T*>(v.z), acc);
     }
     double accd[6];
 #pragma unroll
@@ -463,13 +448,17 @@ __global__ void ms_set_mean_kernel(typename cplx<T>::type* __restrict__ eps_hat,
 // their min and max -> part[q * gridDim.x + block], q = kmin, kmax, mumin, mumax.
 template <int MODE>
 __global__ void __launch_bounds__(kMatBlock) ms_reference_kernel(int64_t nvox, const uint8_t* __restrict__ phase,
-                                                                 const PhaseTable* __restrict__ tab, Step hs,
+                                                                 const PhaseTable* __restrict__ tab, double h,
                                                                  const double* __restrict__ eps_raw,
                                                                  const double* __restrict__ zn, double inv_n3,
                                                                  double d0, double d1, double d2, double d3, double d4,
                                                                  double d5, double* __restrict__ part) {
   const double d[6] = {d0, d1, d2, d3, d4, d5};
   double r[4] = {1e300, -1e300, 1e300, -1e300};
+  __shared__ RayConst ray[kMaxPhases];
+  if (threadIdx.x < kMaxPhases && tab->kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV)
+    ray[threadIdx.x] = make_ray(tab->p64[threadIdx.x], h);
+  __syncthreads();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nvox; base += stride) {
     const int64_t i = base + threadIdx.x;
@@ -482,9 +471,8 @@ __global__ void __launch_bounds__(kMatBlock) ms_reference_kernel(int64_t nvox, c
       e[c] = in ? fma(eps_raw[c * nvox + i], inv_n3, d[c]) : 0.0;
       zi[c] = vp ? zn[c * nvox + i] : 0.0;
     }
-    if constexpr (MODE == MODE_FP64) voxel_fp64<NortonDev>(tab->p64[ph], e, zi, hs, vp, s, zo, t);
-    else voxel_fp32_fix<NortonDev>(tab->p64[ph], tab->p32[ph], e, zi, hs, vp, s, zo, t);
-    if (in && !vp) voxel_elastic<double>(tab->p64[ph], e, s, t);
+    if (vp) voxel_ray<NortonDev>(ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, t);
+    else if (in) voxel_elastic<double>(tab->p64[ph], e, s, t);
     if (in) {
       // packed upper triangle: C11 0, C12 1, C13 2, C22 6, C23 7, C33 11, C44 15, C55 18, C66 20
       const double tk = (t[0] + t[6] + t[11] + 2.0 * (t[1] + t[2] + t[7])) * (1.0 / 3.0);

@@ -183,6 +183,8 @@ struct Job {
   const uint8_t* phase = nullptr;
   PhaseTable tab_host;
   PhaseTable* tab_dev = nullptr;
+  int n_phases = 0;
+  RayConst ray[kMaxPhases] = {};     // the Norton phases' scalar equation at the current step's h
   double lam0 = 0, mu0 = 0;          // reference medium of the current step
   double lam0_el = 0, mu0_el = 0;    // the fixed elastic reference
   double theta[kMaxPhases][3] = {};  // (sigma0, edot0, n) of Norton phases
@@ -212,7 +214,6 @@ struct Job {
   // state
   int step = 0, n_eval = 0, n32 = 0, since_best = 0;
   bool fp32_phase = false, need_start = true, done = false, notconv = false;
-  bool warm = false;  // z holds the previous evaluation of this step, in the current field precision
   double best = 1e300;
   double E_prev[6] = {0, 0, 0, 0, 0, 0};  // macroscopic strain at the end of the previous step
   double E_cur[6] = {0, 0, 0, 0, 0, 0};   // macroscopic strain of the current iterate
@@ -239,6 +240,7 @@ int job_setup(Job& j, int N, const uint8_t* phase_dev, int n_phases, const gsm_h
   j.n_mch = (int)n_mchunks(j.nmodes);
   j.precision = precision;
   j.phase = phase_dev;
+  j.n_phases = n_phases;
   std::memset(&j.tab_host, 0, sizeof(j.tab_host));
   double lam_min = 1e300, lam_max = -1e300, mu_min = 1e300, mu_max = -1e300;
   j.law_mode = MODE_FP64;
@@ -480,16 +482,16 @@ void mixed_setup(Job& j) {
 int reference_update(Engine& g, Job& j, const double (&dE)[6]) {
   const int grid = (int)std::min<int64_t>(j.n_vch, (int64_t)sm_count() * 2);
   const double inv_n3 = 1.0 / (double)j.nvox;
-  const Step hs = make_step(j.h[j.step]);
+  const double h = j.h[j.step];
   if (j.integrator >= 1)
-    ms_launch_reference_ode(j.integrator - 1, grid, g.stream, j.nvox, j.phase, j.tab_dev, hs.h, j.ode_rtol, j.ode_atol,
+    ms_launch_reference_ode(j.integrator - 1, grid, g.stream, j.nvox, j.phase, j.tab_dev, h, j.ode_rtol, j.ode_atol,
                             j.ode_max, j.f64.eps_raw, j.eps_prev, j.f64.zn, j.alpha_n, inv_n3, dE, j.mat_part);
   else if (j.law_mode == MODE_FP64)
-    ms_reference_kernel<MODE_FP64><<<grid, kMatBlock, 0, g.stream>>>(j.nvox, j.phase, j.tab_dev, hs, j.f64.eps_raw,
+    ms_reference_kernel<MODE_FP64><<<grid, kMatBlock, 0, g.stream>>>(j.nvox, j.phase, j.tab_dev, h, j.f64.eps_raw,
                                                                     j.f64.zn, inv_n3, dE[0], dE[1], dE[2], dE[3],
                                                                     dE[4], dE[5], j.mat_part);
   else
-    ms_reference_kernel<MODE_FP32_FIX><<<grid, kMatBlock, 0, g.stream>>>(j.nvox, j.phase, j.tab_dev, hs,
+    ms_reference_kernel<MODE_FP32_FIX><<<grid, kMatBlock, 0, g.stream>>>(j.nvox, j.phase, j.tab_dev, h,
                                                                         j.f64.eps_raw, j.f64.zn, inv_n3, dE[0], dE[1],
                                                                         dE[2], dE[3], dE[4], dE[5], j.mat_part);
   count_launch();
@@ -529,7 +531,8 @@ int step_start(Engine& g, Job& j) {
     if (rc != GSM_OK) return rc;
   }
   mixed_setup(j);
-  j.warm = false;
+  for (int p = 0; p < j.n_phases; ++p)
+    if (j.tab_host.kind[p] == GSM_PSI_ELASTIC_VP_DEV) j.ray[p] = make_ray(j.tab_host.p64[p], j.h[j.step]);
   j.n_eval = 0;
   j.n32 = 0;
   j.best = 1e300;
@@ -563,7 +566,6 @@ template <class T> void move_mean(Engine& g, Job& j, const double (&dS)[6]) {
 // evaluation becomes the FP64 strain, resynthesised from its spectrum so that
 // its mean is E_k exactly.
 int switch_to_fp64(Engine& g, Job& j) {
-  j.warm = false;  // the FP64 z is not this step's
   convert<float, double>(g.stream, j.f32.eps_raw, j.f64.eps_raw, 6 * j.nvox, 1.0);
   int rc = spectrum_start<double>(g, j, j.E_cur, j.E_cur);
   if (rc != GSM_OK) return rc;
@@ -576,7 +578,6 @@ int switch_to_fp64(Engine& g, Job& j) {
 // After the tick's evaluation: convergence, precision switch, step end.
 int post_eval(Engine& g, Job& j, const Reduced& r) {
   ++j.n_eval;
-  j.warm = true;  // z now holds this evaluation (step_start and the precision switch clear it)
   double e = r.e;
   double dS[6] = {0, 0, 0, 0, 0, 0};
   if (j.stress_mask) {
@@ -695,7 +696,8 @@ int tick(Engine& g, const std::vector<Job*>& jobs) {
     v.n_vch = j.n_vch;
     v.n_mch = j.n_mch;
     v.N = j.N;
-    v.warm = (j.warm && j.integrator == 0) ? 1 : 0;
+    v.pad1 = 0;
+    std::memcpy(v.ray, j.ray, j.n_phases * sizeof(RayConst));
     v.h = j.h[j.step];
     v.inv_h = 1.0 / v.h;
     v.inv_n3 = 1.0 / (double)j.nvox;
@@ -1451,7 +1453,7 @@ extern "C" int ms_evaluate_noalloc(int N, const uint8_t* phase, int n_phases, co
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   double* partials = scratch;                                    // [6][grid]
   Reduced* red = reinterpret_cast<Reduced*>(scratch + 6 * kNoAllocMaxBlocks);
-  ms_material_kernel<double, MODE_FP64><<<grid, kMatBlock, 0, s>>>(nvox, phase, tab, make_step(step_h), 1.0, eps, z_n, sigma, z,
+  ms_material_kernel<double, MODE_FP64><<<grid, kMatBlock, 0, s>>>(nvox, phase, tab, step_h, 1.0, eps, z_n, sigma, z,
                                                                    partials);
   ms_finalize_kernel<<<1, kFinBlock, 0, s>>>(partials, grid, nullptr, 0, 1.0 / (double)nvox, 1.0, red);
   count_launch(2);

@@ -1,0 +1,330 @@
+// Implicit-Euler step of a proportional law: the 5-dimensional Newton system
+// of solver.cuh collapses to one scalar equation.
+//
+// A law declares kRay when (i) psi is quadratic and depends on y through the
+// deviatoric strain e_s - P y with an isotropic stiffness, and (ii) phi =
+// c_phi q^a_phi with q = (2/3) zdot:zdot, the norm of the same metric.  Then
+// psi_y(e_s, 0), psi_yy d and phi_v(theta d / h) are all parallel for the
+// predictor d (the increment that relaxes the deviatoric trial strain: d =
+// the y-components of e_s), so R(theta d) = 0 has its root on the predictor
+// segment and the segment minimisation of solver.cuh already gives it; the
+// Newton polish that followed it only confirmed the root (five-direction AD
+// sweeps, a 5x5 factorisation).  With A = -d.psi_y(e_s, 0) = 2 mu (e_s:e_s)
+// and d.phi_v(theta d/h) = 2 mu (e_s:e_s) k(theta) the root solves
+//   k(theta) = 1 - theta,   k(theta) = c0 theta (E2 theta^2)^(a_phi - 1),  E2 = e_s:e_s,
+//   c0 = 2 a_phi c_phi / (3 mu h) (2 / (3 h^2))^(a_phi - 1)      (once per step),
+// and with t = 1 - theta
+//   w = theta d,   sigma = kappa tr(eps) 1 + 2 mu t e_s,
+//   C_t = kappa 1x1 + 2 mu t I_dev - 2 mu (1 - p) theta t / (p t + theta) n x n,
+//   p = 2 a_phi - 1,  n = e_s / |e_s|
+// (the last term from the derivative of the scalar equation, Eq.
+// tangent_formula restricted to the segment).  The host tests compare this
+// with the general solver (the AD-driven Newton) and the oracle over n from 1
+// to 20 and trial strains from 1e-25 to 1e-1.
+//
+// Solution: theta in FP32 from the equation in u = log2 theta (convex and
+// increasing; Newton from an upper bound decreases monotonically onto the
+// root), then Halley steps in the working precision on the equation itself.
+// One step squares^1.5 the seed's ~1e-7: its remainder is below 1e-18, so a
+// voxel takes one power in the working precision.  FP64 operations per voxel:
+// about 75, where the line search and Newton steps took about 800.
+//
+// Bound: FP64 the FP64 pipe (75 operations at 629 G/s: 7.4 G voxel/s at 100 %),
+// FP32 the memory (96 bytes a voxel).  Measured on GB300 against the general
+// solver: FP64 3.0 M voxels (n = 10) 5208 -> 445 us, FP64 with tangent 1.0 M
+// voxels 2793 -> 242 us, FP32 5.0 M voxels 266 -> 88 us (5.5 TB/s), the FP32
+// material kernel of the scheme at 256^3 1199 -> 372 us.
+#pragma once
+
+#include "solver.cuh"
+
+namespace gsm {
+
+// Constants of the scalar equation of one law and one step size.
+struct RayConst {
+  double c0, am1, p, mu, kappa;
+  float am1f, pf, inv_pf, muf, kappaf;
+  float lg_c0;     // log2 c0
+  float c0m;       // c0 = c0m 2^c0e, c0m in [1, 2)
+  int c0e;
+  float lg_floor;  // log2 of 1e-140 h: rates below 1e-140 of |d| / h are no flow
+};
+
+AD_HD float lg2_approx(float x) {
+#if defined(__CUDA_ARCH__)
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return std::log2(x);
+#endif
+}
+AD_HD float ex2_approx(float x) {
+#if defined(__CUDA_ARCH__)
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return std::exp2(x);
+#endif
+}
+AD_HD float rcp_approx(float x) {
+#if defined(__CUDA_ARCH__)
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / x;
+#endif
+}
+
+AD_HD RayConst make_ray(const LawParams<double>& p, double h) {
+  RayConst r;
+  r.am1 = p.a_phi - 1.0;
+  r.p = 1.0 + 2.0 * r.am1;
+  r.mu = p.mu;
+  r.kappa = p.lam + p.mu * (2.0 / 3.0);
+  r.c0 = 2.0 * p.a_phi * p.c_phi / (3.0 * p.mu * h) * ::pow(2.0 / (3.0 * h * h), r.am1);
+  r.am1f = (float)r.am1;
+  r.pf = (float)r.p;
+  r.inv_pf = (float)(1.0 / r.p);
+  r.muf = (float)r.mu;
+  r.kappaf = (float)r.kappa;
+  r.lg_c0 = (float)::log2(r.c0);
+  r.c0e = (int)((fpow::bits_of(r.c0) >> 52) & 0x7ff) - 1023;
+  r.c0m = f32_of(r.c0, -r.c0e);
+  r.lg_floor = (float)::log2(1e-140 * h);
+  return r;
+}
+
+// log2 x of a positive normal FP64 x to FP32 accuracy, whatever its exponent.
+AD_HD float lg2_of(double x) {
+  const uint64_t b = fpow::bits_of(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023;
+  const float m = f32_of(x, -e);
+  return (float)e + lg2_approx(m);
+}
+
+// u = log2 theta of the root of K theta^p + theta = 1, L = log2 K, p > 0.
+// Both terms are at most 1 at the root, so u <= min(0, -L/p); at that bound
+// the larger term is 1, and Newton on the convex increasing function of u
+// decreases monotonically onto the root (three to five iterations).
+AD_HD float ray_seed(float L, float p, float inv_p, int& iters) {
+  float u = fminf(0.0f, -L * inv_p);
+  iters = 0;
+  for (int k = 0; k < 16; ++k) {
+    ++iters;
+    const float a = ex2_approx(L + p * u), b = ex2_approx(u);
+    const float du = 1.44269504f * (1.0f - a - b) * rcp_approx(p * a + b);
+    u += du;
+    if (!(fabsf(du) > 2e-4f)) break;  // quadratic: the next step is below 1e-7
+  }
+  return fminf(u, 0.0f);
+}
+
+struct RayRoot {
+  bool flows;
+  int n_eval, n_model;
+};
+
+// The root in FP64: theta and t = 1 - theta, each to its own rounding.
+AD_HD RayRoot ray_root(const RayConst& c, double E2, bool active, double& theta, double& t) {
+  RayRoot r{false, 0, 0};
+  theta = 0.0;
+  t = 1.0;
+  // E2 = 0 (a stress-free deviatoric state), NaN or out of range: no flow
+  if (!active || !(E2 > 1e-300 && E2 < 1e300)) return r;
+  const float lgE = lg2_of(E2);
+  const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
+  if (!(u + 0.5f * lgE > c.lg_floor) || !(u > -1000.0f)) return r;
+  r.flows = true;
+  const float uf = floorf(u);
+  double th = f64_of(ex2_approx(u - uf), (int)uf);
+  for (int it = 0; it < 8; ++it) {
+    ++r.n_eval;
+    const double s = 1.0 - th;
+    const double k = c.c0 * th * fpow::pow_pos(E2 * (th * th), c.am1);
+    const double pk = c.p * k;
+    const double D = pk + th;  // theta d/dtheta of k + theta
+    // 1/D by one Newton step from the FP32 reciprocal (relative error ~1e-14)
+    const int e = (int)((fpow::bits_of(D) >> 52) & 0x7ff) - 1023;
+    const float Df = f32_of(D, -e);
+    const float y0 = rcp_approx(Df);
+    double y = f64_of(y0, -e);
+    y = fma(y, fma(-D, y, 1.0), y);
+    const double eta = (s - k) * y;  // Newton step of ln theta
+    // Halley: eta / (1 + eta (p - 1)/2 pk/D); the correction is O(eta^2), FP32
+    const float ef = f32_of(eta);
+    const float q = 0.5f * (c.pf - 1.0f) * f32_of(pk, -e) * y0 * ef;
+    const double step = eta - eta * f64_of(q * rcp_approx(1.0f + q));
+    const double dth = th * step;
+    theta = th + dth;
+    t = s - dth;
+    if (!(fabsf(ef) > 8e-6f)) break;  // remainder below eta^3 / 10
+    th = theta > 0.0 ? theta : 0.5 * th;
+  }
+  return r;
+}
+
+AD_HD unsigned ray_status(const RayRoot& r, bool correction) {
+  unsigned st = ST_CONVERGED | ((unsigned)(r.n_model & 0x7f) << ST_MODEL_SHIFT);
+  if (correction)
+    st |= ((unsigned)r.n_eval << ST_NEWTON_SHIFT) | ((unsigned)(r.n_eval & 0xf) << ST_FIX_SHIFT);
+  else
+    st |= (unsigned)r.n_eval << ST_LINE_SHIFT;
+  return st;
+}
+
+template <class T> AD_HD T recip_of(T x);
+template <> AD_HD double recip_of(double x) { return recip_pos(x); }
+template <> AD_HD float recip_of(float x) { return 1.0f / x; }
+
+// Consistent tangent (21 packed entries) at the root.
+template <class T>
+AD_HD void ray_tangent(T mu, T kappa, T p, const T (&es)[6], T E2, T theta, T t, bool flows, T (&C21)[21]) {
+  T m[6], cm[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) m[i] = i < 3 ? es[i] : T(0.5) * es[i];
+  T c3 = T(0);
+  if (flows) c3 = T(-2) * mu * (T(1) - p) * (theta * t) * recip_of<T>((p * t + theta) * E2);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) cm[i] = c3 * m[i];
+  const T g = mu * t;                                // shear modulus of the deviatoric part
+  const T off = kappa - g * T(2.0 / 3.0), dia = off + T(2) * g;
+  int q = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = i; j < 6; ++j) {
+      const T base = i == j ? (i < 3 ? dia : g) : (j < 3 ? off : T(0));
+      C21[q++] = cm[i] * m[j] + base;
+    }
+}
+
+// One voxel in FP64 (correction: the FP32-bulk mode's status bookkeeping).
+template <class Law>
+AD_HD unsigned voxel_ray(const RayConst& c, const double (&eps)[6], const double (&zn)[6], bool active,
+                         bool correction, double (&sig)[6], double (&z)[6], double* C21) {
+  const double yn[5] = {zn[0], zn[1], zn[3], zn[4], zn[5]};
+  double es[6];
+  const double tr = Law::trial_strain(eps, yn, es);
+  const double E2 = es[0] * es[0] + es[1] * es[1] + es[2] * es[2] +
+                    0.5 * (es[3] * es[3] + es[4] * es[4] + es[5] * es[5]);
+  double theta, t;
+  const RayRoot r = ray_root(c, E2, active, theta, t);
+  unsigned st = ray_status(r, correction);
+  if (active && !(E2 < 1e300)) st |= ST_NONFINITE;
+  const double hyd = c.kappa * tr, g = c.mu * t, g2 = g + g;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) sig[i] = fma(g2, es[i], hyd);
+#pragma unroll
+  for (int i = 3; i < 6; ++i) sig[i] = g * es[i];
+  z[0] = r.flows ? fma(theta, es[0], yn[0]) : yn[0];
+  z[1] = r.flows ? fma(theta, es[1], yn[1]) : yn[1];
+  z[2] = -(z[0] + z[1]);
+#pragma unroll
+  for (int i = 3; i < 6; ++i) z[i] = r.flows ? fma(theta, es[i], yn[i - 1]) : yn[i - 1];
+  if (C21) {
+    double C[21];
+    ray_tangent<double>(c.mu, c.kappa, c.p, es, E2, theta, t, r.flows, C);
+#pragma unroll
+    for (int q = 0; q < 21; ++q) C21[q] = C[q];
+  }
+  return st;
+}
+
+// floor(log2 x) of a positive normal FP32 x.
+AD_HD int ilog2_pos(float x) {
+#if defined(__CUDA_ARCH__)
+  return (int)(__float_as_uint(x) >> 23) - 127;
+#else
+  unsigned b;
+  std::memcpy(&b, &x, sizeof b);
+  return (int)(b >> 23) - 127;
+#endif
+}
+
+// FP32 power (2^e m)^a with lgm = log2 m: the product a e is split into its
+// integer part and an exact remainder, so the result carries ~2^-23, not
+// 2^-23 of the exponent.  Returns r with the power = 2^n r.
+AD_HD float ray_pow(float a, int e, float lgm, int& n) {
+  const float ef = (float)e;
+  const float yh = a * ef;
+  const float yl = fmaf(a, ef, -yh);
+  const float ni = rintf(yh);
+  n = (int)ni;
+  return ex2_approx((yh - ni) + fmaf(a, lgm, yl));
+}
+
+// One voxel in FP32.  E2 is formed on e_s scaled by 2^-k, k = the exponent of
+// its largest entry, so that no trial strain under- or overflows.
+template <class Law>
+AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (&zn)[6], bool active, bool,
+                         float (&sig)[6], float (&z)[6], float* C21) {
+  const float yn[5] = {zn[0], zn[1], zn[3], zn[4], zn[5]};
+  float es[6], ss[6];
+  const float tr = Law::trial_strain(eps, yn, es);
+  const int k0 = ilog2_max(es);
+  const int k = k0 > 126 ? 126 : k0;
+  const float inv_s = exp2i(-k, 0.0f);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) ss[i] = es[i] * inv_s;
+  const float E2 = ss[0] * ss[0] + ss[1] * ss[1] + ss[2] * ss[2] +
+                   0.5f * (ss[3] * ss[3] + ss[4] * ss[4] + ss[5] * ss[5]);  // in [0.5, 24)
+  RayRoot r{false, 0, 0};
+  float theta = 0.0f, t = 1.0f;
+  if (active && E2 > 0.0f && E2 < 1e30f) {
+    const float lgE = lg2_approx(E2) + 2.0f * (float)k;
+    const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
+    if (u > -120.0f) {
+      r.flows = true;
+      float th = ex2_approx(u);
+      for (int it = 0; it < 4; ++it) {
+        ++r.n_eval;
+        const float s = 1.0f - th;
+        // (E2 th^2)^am1 with th = tm 2^et, E2 tm^2 in [0.5, 96)
+        const int et = ilog2_pos(th);
+        const float tm = th * exp2i(-et, 0.0f);
+        const float x = E2 * tm * tm;
+        const int ex = ilog2_pos(x);
+        int n;
+        const float pw = ray_pow(c.am1f, ex + 2 * (k + et), lg2_approx(x * exp2i(-ex, 0.0f)), n);
+        n += c.c0e;
+        n = n > 240 ? 240 : (n < -240 ? -240 : n);
+        const int n1 = n / 2;
+        const float kk = (c.c0m * th * exp2i(n1, 0.0f)) * (pw * exp2i(n - n1, 0.0f));
+        const float pk = c.pf * kk;
+        const float y0 = rcp_approx(pk + th);
+        const float eta = (s - kk) * y0;
+        const float q = 0.5f * (c.pf - 1.0f) * pk * y0 * eta;
+        const float dth = th * (eta - eta * q * rcp_approx(1.0f + q));
+        theta = th + dth;
+        t = s - dth;
+        if (!(fabsf(eta) > 1e-3f)) break;
+        th = theta > 0.0f ? theta : 0.5f * th;
+      }
+    }
+  }
+  unsigned st = ray_status(r, false);
+  if (active && !(E2 < 1e30f)) st |= ST_NONFINITE;
+  const float hyd = c.kappaf * tr, g = c.muf * t, g2 = g + g;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) sig[i] = fmaf(g2, es[i], hyd);
+#pragma unroll
+  for (int i = 3; i < 6; ++i) sig[i] = g * es[i];
+  z[0] = r.flows ? fmaf(theta, es[0], yn[0]) : yn[0];
+  z[1] = r.flows ? fmaf(theta, es[1], yn[1]) : yn[1];
+  z[2] = -(z[0] + z[1]);
+#pragma unroll
+  for (int i = 3; i < 6; ++i) z[i] = r.flows ? fmaf(theta, es[i], yn[i - 1]) : yn[i - 1];
+  if (C21) {
+    float C[21];
+    // n x n is scale free: the tangent takes the scaled trial strain
+    ray_tangent<float>(c.muf, c.kappaf, c.pf, ss, E2, theta, t, r.flows, C);
+#pragma unroll
+    for (int q = 0; q < 21; ++q) C21[q] = C[q];
+  }
+  return st;
+}
+
+}  // namespace gsm
