@@ -17,7 +17,9 @@
 // About 26 FP64 operations and three L1-resident table loads; the result is
 // within a few ulp of x^p (checked against a 50-digit reference on the host
 // and against CUDA's pow on the GPU).  Zero, subnormal, negative and
-// non-finite x, and |p log2 x| >= 1000, take CUDA's pow.
+// non-finite x, and |p log2 x| >= 512, take CUDA's pow.  Range tests and the
+// exponent's conversion are integer operations (an FP64 compare or conversion
+// occupies the FP64 pipe).
 #pragma once
 
 #include <cmath>
@@ -71,6 +73,17 @@ AD_HD double double_of(uint64_t b) {
 #endif
 }
 
+// The double equal to the integer j, |j| < 2^24, by integer operations.
+AD_HD double double_of_int(int j) {
+#if defined(__CUDA_ARCH__)
+  const unsigned f = __float_as_uint((float)j);
+  const uint64_t m = (uint64_t)(f & 0x7fffffffu) << 29;
+  return double_of((m ? m + ((uint64_t)896 << 52) : 0) | ((uint64_t)(f & 0x80000000u) << 32));
+#else
+  return (double)j;
+#endif
+}
+
 AD_HD double pow_pos(double x, double p) {
   const uint64_t b = bits_of(x);
   const int e = (int)((b >> 52) & 0x7ff);
@@ -84,10 +97,10 @@ AD_HD double pow_pos(double x, double p) {
 #pragma unroll
   for (int k = 5; k >= 0; --k) s = fma(s, t, GSM_POW_TAB(kPowLnC, k));
   const double l = fma(s, t, GSM_POW_TAB(kPowLog2, i));  // log2 m in [0, 1)
-  const double jd = (double)j;
+  const double jd = double_of_int(j);
   const double yj = p * jd;
   const double yl = fma(p, l, fma(p, jd, -yj));  // y = yj + yl
-  if (!(yj < 1000.0 && yj > -1000.0)) return ::pow(x, p);
+  if (((bits_of(yj) >> 52) & 0x7ff) >= 1023 + 9) return ::pow(x, p);  // |y| >= 512 or not finite
   const double magic = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer
   const double sh = fma(yj + yl, 128.0, magic);
   const int64_t n = (int64_t)(bits_of(sh) - bits_of(magic));

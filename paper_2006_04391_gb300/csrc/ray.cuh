@@ -31,11 +31,14 @@
 //
 // Bound: FP64 the FP64 pipe (75 operations at 629 G/s: 7.4 G voxel/s at 100 %),
 // FP32 the memory (96 bytes a voxel).  Measured on GB300 against the general
-// solver: FP64 3.0 M voxels (n = 10) 5208 -> 445 us, FP64 with tangent 1.0 M
-// voxels 2793 -> 242 us, FP32 5.0 M voxels 266 -> 88 us (5.5 TB/s), the FP32
+// solver: FP64 3.0 M voxels (n = 10) 5208 -> 415 us (97 % of the FP64 pipe's
+// issue rate for these operations), FP64 with tangent 1.0 M voxels 2793 -> 232
+// us, FP32 5.0 M voxels 266 -> 87 us (5.5 TB/s), FP32 bulk + correction 2^24
+// voxels 3015 -> 1119 us (2450 with the correction in FP64; 2.9 TB/s), the FP32
 // material kernel of the scheme at 256^3 1199 -> 372 us.
 #pragma once
 
+#include "dpow.cuh"
 #include "solver.cuh"
 
 namespace gsm {
@@ -48,6 +51,7 @@ struct RayConst {
   float c0m;       // c0 = c0m 2^c0e, c0m in [1, 2)
   int c0e;
   float lg_floor;  // log2 of 1e-140 h: rates below 1e-140 of |d| / h are no flow
+  df am1d, pd, c0d;  // am1, p and c0 2^-c0e as double-float pairs (the FP32-bulk correction)
 };
 
 AD_HD float lg2_approx(float x) {
@@ -78,6 +82,17 @@ AD_HD float rcp_approx(float x) {
 #endif
 }
 
+// floor(log2 x) of a positive normal FP32 x.
+AD_HD int ilog2_pos(float x) {
+#if defined(__CUDA_ARCH__)
+  return (int)(__float_as_uint(x) >> 23) - 127;
+#else
+  unsigned b;
+  std::memcpy(&b, &x, sizeof b);
+  return (int)(b >> 23) - 127;
+#endif
+}
+
 AD_HD RayConst make_ray(const LawParams<double>& p, double h) {
   RayConst r;
   r.am1 = p.a_phi - 1.0;
@@ -94,6 +109,9 @@ AD_HD RayConst make_ray(const LawParams<double>& p, double h) {
   r.c0e = (int)((fpow::bits_of(r.c0) >> 52) & 0x7ff) - 1023;
   r.c0m = f32_of(r.c0, -r.c0e);
   r.lg_floor = (float)::log2(1e-140 * h);
+  r.am1d = df_of(r.am1);
+  r.pd = df_of(r.p);
+  r.c0d = df_of(r.c0, -r.c0e);
   return r;
 }
 
@@ -123,17 +141,19 @@ AD_HD float ray_seed(float L, float p, float inv_p, int& iters) {
 }
 
 struct RayRoot {
-  bool flows;
+  bool flows, bad;  // bad: the trial strain is not finite
   int n_eval, n_model;
 };
 
 // The root in FP64: theta and t = 1 - theta, each to its own rounding.
 AD_HD RayRoot ray_root(const RayConst& c, double E2, bool active, double& theta, double& t) {
-  RayRoot r{false, 0, 0};
+  RayRoot r{false, false, 0, 0};
   theta = 0.0;
   t = 1.0;
   // E2 = 0 (a stress-free deviatoric state), NaN or out of range: no flow
-  if (!active || !(E2 > 1e-300 && E2 < 1e300)) return r;
+  const int e2 = (int)((fpow::bits_of(E2) >> 52) & 0x7ff);
+  r.bad = active && e2 > 1023 + 996;
+  if (!active || e2 < 1023 - 996 || r.bad) return r;
   const float lgE = lg2_of(E2);
   const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
   if (!(u + 0.5f * lgE > c.lg_floor) || !(u > -1000.0f)) return r;
@@ -166,8 +186,84 @@ AD_HD RayRoot ray_root(const RayConst& c, double E2, bool active, double& theta,
   return r;
 }
 
+// x 2^k as a double-float pair by integer operations alone: hi is x truncated
+// to FP32, lo the 29 mantissa bits below it.
+AD_HD df df_bits(double x, int k) {
+  const uint64_t b = fpow::bits_of(x);
+  const float lo = (float)(int)(b & 0x1fffffffu);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023 - 52 + k;
+  const float sc = e < -126 ? 0.0f : exp2i(e, 0.0f);
+  return df{f32_of(x, k), (b >> 63) ? -lo * sc : lo * sc};
+}
+
+// The root of the FP32-bulk mode: FP32 seed, then the Halley step with the
+// equation's residual in double-float arithmetic (2^-45, the accuracy of this
+// mode's correction), on e_s scaled by 2^-k.  FP64 operations: three inside the
+// power and one per result, where ray_root takes about 45; the FP64 pipe runs
+// at 1/64 of the FP32 rate.  Returns false where a value leaves the pairs'
+// range (the caller takes ray_root).
+AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool active, RayRoot& r, double& theta,
+                       double& t) {
+  r = RayRoot{false, false, 0, 0};
+  theta = 0.0;
+  t = 1.0;
+  if (!active) return true;
+  // E2 = e_s:e_s, scaled: squares of the pairs, normal and shear parts apart
+  df n, h;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const df a = df_bits(es[i], -k);
+    const float p = dfo::mul_rn(a.hi, a.hi);
+    const float q = dfo::fma_rn(a.hi + a.hi, a.lo, dfo::fma_rn(a.hi, a.hi, -p));
+    df& s = i < 3 ? n : h;
+    if (i % 3 == 0) {
+      s = df{p, q};
+    } else {
+      const df u = dfo::two_sum(s.hi, p);
+      s = df{u.hi, dfo::add_rn(s.lo, dfo::add_rn(u.lo, q))};
+    }
+  }
+  const df u2 = dfo::two_sum(n.hi, 0.5f * h.hi);
+  const df E2 = dfo::fast_two_sum(u2.hi, dfo::add_rn(u2.lo, dfo::fma_rn(0.5f, h.lo, n.lo)));
+  if (!(E2.hi > 0.25f && E2.hi < 64.0f)) return false;  // zero, non-finite or subnormal trial strain
+  const float lgE = lg2_approx(E2.hi) + 2.0f * (float)k;
+  const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
+  if (!(u > -40.0f)) return false;
+  float th = ex2_approx(u);
+  for (int it = 0; it < 8; ++it) {
+    ++r.n_eval;
+    const int et = ilog2_pos(th);
+    const float tm = th * exp2i(-et, 0.0f);
+    const float t2 = dfo::mul_rn(tm, tm);
+    const df x = E2 * df{t2, dfo::fma_rn(tm, tm, -t2)};
+    df F;
+    if (!dpow::pow_scaled(x, 2 * (k + et), c.am1, c.am1d, c.c0d, c.c0e, F)) return false;
+    const df kk = F * th;
+    const df s = dfo::two_sum(1.0f, -th);
+    const df R = s - kk;
+    const df D = kk * c.pd + th;
+    // eta = R / D as a pair, then Halley's factor (FP32: second order)
+    const float y0 = rcp_approx(D.hi);
+    const float eta = R.hi * y0;
+    const float q = 0.5f * (c.pf - 1.0f) * c.pf * kk.hi * y0 * eta;
+    const float rest = dfo::fma_rn(-eta, D.hi, R.hi) + dfo::fma_rn(-eta, D.lo, R.lo);
+    const df step = dfo::fast_two_sum(eta, dfo::fma_rn(rest, y0, -eta * q * rcp_approx(1.0f + q)));
+    const df dth = step * th;
+    if (!(fabsf(eta) > 8e-6f)) {
+      theta = f64_of(dth + th);
+      t = f64_of(s - dth);
+      r.flows = true;
+      return true;
+    }
+    th = th + dth.hi;
+    if (!(th > 1e-12f)) return false;
+  }
+  return false;
+}
+
 AD_HD unsigned ray_status(const RayRoot& r, bool correction) {
   unsigned st = ST_CONVERGED | ((unsigned)(r.n_model & 0x7f) << ST_MODEL_SHIFT);
+  if (r.bad) st |= ST_NONFINITE;
   if (correction)
     st |= ((unsigned)r.n_eval << ST_NEWTON_SHIFT) | ((unsigned)(r.n_eval & 0xf) << ST_FIX_SHIFT);
   else
@@ -201,47 +297,91 @@ AD_HD void ray_tangent(T mu, T kappa, T p, const T (&es)[6], T E2, T theta, T t,
     }
 }
 
-// One voxel in FP64 (correction: the FP32-bulk mode's status bookkeeping).
+// Trial state and root of one voxel in FP64 (correction: the FP32-bulk mode).
+struct RayVoxel {
+  double es[6], tr, theta, t;
+  RayRoot r;
+  AD_HD double norm2() const {
+    return es[0] * es[0] + es[1] * es[1] + es[2] * es[2] + 0.5 * (es[3] * es[3] + es[4] * es[4] + es[5] * es[5]);
+  }
+};
 template <class Law>
-AD_HD unsigned voxel_ray(const RayConst& c, const double (&eps)[6], const double (&zn)[6], bool active,
-                         bool correction, double (&sig)[6], double (&z)[6], double* C21) {
-  const double yn[5] = {zn[0], zn[1], zn[3], zn[4], zn[5]};
-  double es[6];
-  const double tr = Law::trial_strain(eps, yn, es);
-  const double E2 = es[0] * es[0] + es[1] * es[1] + es[2] * es[2] +
-                    0.5 * (es[3] * es[3] + es[4] * es[4] + es[5] * es[5]);
-  double theta, t;
-  const RayRoot r = ray_root(c, E2, active, theta, t);
-  unsigned st = ray_status(r, correction);
-  if (active && !(E2 < 1e300)) st |= ST_NONFINITE;
+AD_HD void ray_solve(const RayConst& c, const double (&eps)[6], const double (&yn)[5], bool active, bool correction,
+                     RayVoxel& v) {
+  v.tr = Law::trial_strain(eps, yn, v.es);
+  if (!correction || !ray_root_df(c, v.es, ilog2_max(v.es), active, v.r, v.theta, v.t))
+    v.r = ray_root(c, v.norm2(), active, v.theta, v.t);
+}
+AD_HD void ray_stress(const RayConst& c, const double (&es)[6], double tr, double t, double (&sig)[6]) {
   const double hyd = c.kappa * tr, g = c.mu * t, g2 = g + g;
 #pragma unroll
   for (int i = 0; i < 3; ++i) sig[i] = fma(g2, es[i], hyd);
 #pragma unroll
   for (int i = 3; i < 6; ++i) sig[i] = g * es[i];
-  z[0] = r.flows ? fma(theta, es[0], yn[0]) : yn[0];
-  z[1] = r.flows ? fma(theta, es[1], yn[1]) : yn[1];
+}
+
+// One voxel in FP64 (correction: the FP32-bulk mode and its status bookkeeping).
+template <class Law>
+AD_HD unsigned voxel_ray(const RayConst& c, const double (&eps)[6], const double (&zn)[6], bool active,
+                         bool correction, double (&sig)[6], double (&z)[6], double* C21) {
+  const double yn[5] = {zn[0], zn[1], zn[3], zn[4], zn[5]};
+  RayVoxel v;
+  ray_solve<Law>(c, eps, yn, active, correction, v);
+  ray_stress(c, v.es, v.tr, v.t, sig);
+  const bool flows = v.r.flows;
+  z[0] = flows ? fma(v.theta, v.es[0], yn[0]) : yn[0];
+  z[1] = flows ? fma(v.theta, v.es[1], yn[1]) : yn[1];
   z[2] = -(z[0] + z[1]);
 #pragma unroll
-  for (int i = 3; i < 6; ++i) z[i] = r.flows ? fma(theta, es[i], yn[i - 1]) : yn[i - 1];
+  for (int i = 3; i < 6; ++i) z[i] = flows ? fma(v.theta, v.es[i], yn[i - 1]) : yn[i - 1];
   if (C21) {
     double C[21];
-    ray_tangent<double>(c.mu, c.kappa, c.p, es, E2, theta, t, r.flows, C);
+    ray_tangent<double>(c.mu, c.kappa, c.p, v.es, v.norm2(), v.theta, v.t, flows, C);
 #pragma unroll
     for (int q = 0; q < 21; ++q) C21[q] = C[q];
   }
-  return st;
+  return ray_status(v.r, correction);
 }
 
-// floor(log2 x) of a positive normal FP32 x.
-AD_HD int ilog2_pos(float x) {
-#if defined(__CUDA_ARCH__)
-  return (int)(__float_as_uint(x) >> 23) - 127;
-#else
-  unsigned b;
-  std::memcpy(&b, &x, sizeof b);
-  return (int)(b >> 23) - 127;
-#endif
+// The Newton matrix at the root, K = psi_yy + phi_vv / h, in the metric M of the
+// y coordinates (z:z = y^T M y) and d, the y components of e_s:
+//   K = (2 mu / theta) (M + t (p - 1)/E2 (M d)(M d)^T),
+//   phi_vv / h = K - 2 mu M = (2 mu t / theta) (M + (p - 1)/E2 (M d)(M d)^T),
+// for the adjoint: K^-1 by Sherman and Morrison, no factorisation.
+AD_HD void metric_apply(const double (&y)[5], double (&out)[5]) {
+  const double s = y[0] + y[1];
+  out[0] = y[0] + s;
+  out[1] = y[1] + s;
+  out[2] = 0.5 * y[2];
+  out[3] = 0.5 * y[3];
+  out[4] = 0.5 * y[4];
+}
+// b = K^-1 g
+AD_HD void ray_K_solve(double mu, double p, double theta, double t, double E2, const double (&d)[5],
+                       const double (&g)[5], double (&b)[5]) {
+  const double f = theta / (2.0 * mu);
+  double dg = 0.0;
+#pragma unroll
+  for (int a = 0; a < 5; ++a) dg += d[a] * g[a];
+  const double w = t * (1.0 - p) * dg / (E2 * (theta + p * t));
+  const double m = (g[0] + g[1]) * (1.0 / 3.0);
+  b[0] = f * ((g[0] - m) + w * d[0]);
+  b[1] = f * ((g[1] - m) + w * d[1]);
+#pragma unroll
+  for (int a = 2; a < 5; ++a) b[a] = f * (2.0 * g[a] + w * d[a]);
+}
+// out = (phi_vv / h) b
+AD_HD void ray_flow_apply(double mu, double p, double theta, double t, double E2, const double (&d)[5],
+                          const double (&b)[5], double (&out)[5]) {
+  double Mb[5], Md[5];
+  metric_apply(b, Mb);
+  metric_apply(d, Md);
+  double db = 0.0;
+#pragma unroll
+  for (int a = 0; a < 5; ++a) db += d[a] * Mb[a];
+  const double f = 2.0 * mu * t / theta, w = (p - 1.0) * db / E2;
+#pragma unroll
+  for (int a = 0; a < 5; ++a) out[a] = f * (Mb[a] + w * Md[a]);
 }
 
 // FP32 power (2^e m)^a with lgm = log2 m: the product a e is split into its
@@ -271,7 +411,7 @@ AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (
   for (int i = 0; i < 6; ++i) ss[i] = es[i] * inv_s;
   const float E2 = ss[0] * ss[0] + ss[1] * ss[1] + ss[2] * ss[2] +
                    0.5f * (ss[3] * ss[3] + ss[4] * ss[4] + ss[5] * ss[5]);  // in [0.5, 24)
-  RayRoot r{false, 0, 0};
+  RayRoot r{false, active && !(E2 < 1e30f), 0, 0};
   float theta = 0.0f, t = 1.0f;
   if (active && E2 > 0.0f && E2 < 1e30f) {
     const float lgE = lg2_approx(E2) + 2.0f * (float)k;
@@ -306,7 +446,6 @@ AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (
     }
   }
   unsigned st = ray_status(r, false);
-  if (active && !(E2 < 1e30f)) st |= ST_NONFINITE;
   const float hyd = c.kappaf * tr, g = c.muf * t, g2 = g + g;
 #pragma unroll
   for (int i = 0; i < 3; ++i) sig[i] = fmaf(g2, es[i], hyd);
