@@ -3,7 +3,7 @@
 // ms_solve.cu and (for the job views and block reductions) ms_ode.cu.
 //
 // Every kernel works on a batch of independent problems ("jobs") at once: a
-// job's voxels (modes) are cut into fixed chunks of kVChunk (kMChunk), the
+// job's voxels (modes) are cut into chunks of a size fixed by its grid, the
 // chunks of all jobs in a launch are numbered consecutively, and each block
 // walks the global chunk list.  Partial sums are written per chunk and summed
 // per job in chunk order, so a job's results are bit-identical whether it
@@ -29,7 +29,7 @@ namespace {
 constexpr int kMaxPhases = 16;
 constexpr int kMatBlock = 128;
 constexpr int kGamBlock = 256;
-constexpr int kVChunk = 1024;  // voxels per chunk (8 sweeps of a material block)
+constexpr int kVChunk = 1024;  // largest voxel chunk (8 sweeps of a material block)
 constexpr int kMChunk = 2048;  // modes per chunk (8 sweeps of a gamma block)
 constexpr int kMaxBatch = 256; // jobs per launch
 constexpr double kTwoPi = 6.283185307179586476925286766559;
@@ -44,6 +44,10 @@ template <class T> struct cplx;
 template <> struct cplx<double> { using type = cufftDoubleComplex; };
 template <> struct cplx<float> { using type = cufftComplex; };
 
+struct double6 {
+  double v[6];
+};
+
 struct Reduced {
   double e;        // equilibrium error
   double mean[6];  // <sigma>
@@ -53,22 +57,29 @@ struct Reduced {
 // One job of a batched launch (device copy, rebuilt by the host every tick).
 struct JobView {
   RayConst ray[kMaxPhases];  // the scalar equation of each Norton phase at this step's h
+  int kind[kMaxPhases];      // GSM_PSI_* of each phase
   const uint8_t* phase;
   const void* eps_raw;   // [6][nvox] N^3 * strain (C2R output)
   const void* zn;        // [6][nvox]
   void* sig;             // [6][nvox]
+  void* eps_out;         // [6][nvox] where the inverse transform writes the next strain
   void* z;               // [6][nvox]
   void* sig_hat;         // [6][nmodes]
   void* eps_hat;         // [6][nmodes]
   double* mat_part;      // [6][n_vch]
   double* gam_part;      // [n_mch]
+  Reduced* red;          // where the job's error and mean stress go (page-locked host memory)
+  unsigned* arrived;     // blocks of the fused Green pass that are done (0 between launches), or NULL
   const PhaseTable* tab;
   int64_t nvox, nmodes;
   int64_t vchunk0, mchunk0;  // first chunk of this job in its launch
   int n_vch, n_mch;
   int N;
-  int pad1;
+  int chunk;             // voxels per chunk
+  int project;           // 1: the Green pass gives -Gamma0 : sig_hat alone, eps_hat is not used (adjoint)
+  int n_phases;
   double h, inv_h, inv_n3, lam0, mu0;
+  double inv4mu, green_b;  // constants of the fused Green pass (fft.cuh), set_reference
   // ode23 laws (Sec. 4.3): strain at t_n, the Michel-Suquet alpha, tolerances
   const double* eps_prev;  // [6][nvox]
   const double* alpha_n;   // [nvox] or NULL
@@ -76,6 +87,13 @@ struct JobView {
   double ode_rtol, ode_atol;
   int ode_max, pad2;
 };
+
+inline void set_reference(JobView& v, double lam0, double mu0) {
+  v.lam0 = lam0;
+  v.mu0 = mu0;
+  v.inv4mu = 0.25 / mu0;
+  v.green_b = 0.25 * (lam0 + mu0) / (mu0 * (lam0 + 2.0 * mu0));
+}
 
 // ------------------------------------------------------------------ helpers
 
@@ -110,23 +128,67 @@ template <int NV> __device__ void block_sum(double (&v)[NV], double* out, int64_
   block_sum_at<NV>(v, out, stride, blockIdx.x);
 }
 
+// Block-wide deterministic sum of six FP64 values a lane, as block_sum_at<6>: the
+// lanes of a warp split the components between them as they combine (9 FP64
+// additions a warp instead of 30, 18 shuffles instead of 60; an FP64 warp
+// instruction holds the SM's FP64 pipe for 16 cycles).
+__device__ __forceinline__ void block_sum6_at(const double (&v)[6], double* out, int64_t stride, int64_t index) {
+  __shared__ double sh[6][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+  double a[4], b[2], c;  // lanes with bit 4: components 4, 5; else 0..3
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double lo = v[k], hi = k < 2 ? v[4 + k] : 0.0;
+    const double r = __shfl_xor_sync(0xffffffffu, h16 ? lo : hi, 16);
+    a[k] = (h16 ? hi : lo) + r;
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double r = __shfl_xor_sync(0xffffffffu, h8 ? a[k] : a[2 + k], 8);
+    b[k] = (h8 ? a[2 + k] : a[k]) + r;
+  }
+  c = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  const int comp = (h16 ? 4 : 0) + (h8 ? 2 : 0) + (h4 ? 1 : 0);
+  if ((lane & 3) == 0 && comp < 6) sh[comp][warp] = c;
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    const int nw = blockDim.x >> 5;
+    double s = 0.0;
+    for (int w = 0; w < nw; ++w) s += sh[threadIdx.x][w];
+    out[threadIdx.x * stride + index] = s;
+  }
+  __syncthreads();
+}
+
+// The laws of a job's phases as the material kernels read them (shared memory).
+struct LawTable {
+  RayConst ray[kMaxPhases];
+  int kind[kMaxPhases];
+};
+
 // Material evaluation of voxel i.  The field precision T is also that of the
 // 1/N^3 scaling and of the lane's partial stress sums (FP32 fields: no FP64
 // work, a sixty-fourth of the FP32 rate on GB300; the block sums are FP64).
+// All loads are issued before the phase is known: z_n of an elastic voxel is
+// read for nothing, but no load waits for another.
 template <class T, int MODE>
 __device__ __forceinline__ void material_voxel(int64_t i, int64_t nvox, const uint8_t* __restrict__ phase,
-                                               const PhaseTable& tab, const RayConst* ray, T inv_n3,
+                                               const PhaseTable& tab, const LawTable& law, T inv_n3,
                                                const T* __restrict__ eps_raw, const T* __restrict__ zn,
                                                T* __restrict__ sig, T* __restrict__ z, T (&acc)[6]) {
-  const int ph = (int)phase[i];
-  T e[6], s[6], zo[6] = {0, 0, 0, 0, 0, 0};
+  const int ph = (int)__ldg(phase + i);
+  T e[6], zi[6], s[6], zo[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
-  for (int c = 0; c < 6; ++c) e[c] = __ldg(eps_raw + c * nvox + i) * inv_n3;
-  if (tab.kind[ph] == GSM_PSI_ELASTIC_VP_DEV) {
-    T zi[6];
+  for (int c = 0; c < 6; ++c) e[c] = __ldg(eps_raw + c * nvox + i);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) zi[c] = __ldg(zn + c * nvox + i);
-    voxel_ray<NortonDev>(ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<T*>(nullptr));
+  for (int c = 0; c < 6; ++c) zi[c] = __ldg(zn + c * nvox + i);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) e[c] *= inv_n3;
+  if (law.kind[ph] == GSM_PSI_ELASTIC_VP_DEV) {
+    voxel_ray<NortonDev>(law.ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<T*>(nullptr));
   } else {
     if constexpr (sizeof(T) == 8) voxel_elastic<double>(tab.p64[ph], e, s, nullptr);
     else voxel_elastic<float>(tab.p32[ph], e, s, nullptr);
@@ -297,18 +359,20 @@ __global__ void __launch_bounds__(kMatBlock) ms_material_kernel(int64_t nvox, co
                                                                 const T* __restrict__ eps_raw,
                                                                 const T* __restrict__ zn, T* __restrict__ sig,
                                                                 T* __restrict__ z, double* __restrict__ partials) {
-  __shared__ RayConst ray[kMaxPhases];
-  if (threadIdx.x < kMaxPhases && tab.kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV)
-    ray[threadIdx.x] = make_ray(tab.p64[threadIdx.x], h);
+  __shared__ LawTable law;
+  if (threadIdx.x < kMaxPhases) {
+    law.kind[threadIdx.x] = tab.kind[threadIdx.x];
+    if (tab.kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV) law.ray[threadIdx.x] = make_ray(tab.p64[threadIdx.x], h);
+  }
   __syncthreads();
   T acc[6] = {0, 0, 0, 0, 0, 0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += stride)
-    material_voxel<T, MODE>(i, nvox, phase, tab, ray, (T)inv_n3, eps_raw, zn, sig, z, acc);
+    material_voxel<T, MODE>(i, nvox, phase, tab, law, (T)inv_n3, eps_raw, zn, sig, z, acc);
   double accd[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) accd[c] = (double)acc[c];
-  block_sum<6>(accd, partials, gridDim.x);
+  block_sum6_at(accd, partials, gridDim.x, blockIdx.x);
 }
 
 // Index of the job owning global chunk c (starts ascending, starts[0] = 0).
@@ -326,23 +390,35 @@ template <class T, int MODE>
 __global__ void __launch_bounds__(kMatBlock) ms_material_batch_kernel(const JobView* __restrict__ views, int n_jobs,
                                                                       int64_t total_chunks) {
   __shared__ int64_t starts[kMaxBatch];
+  __shared__ LawTable law;
   for (int j = threadIdx.x; j < n_jobs; j += blockDim.x) starts[j] = views[j].vchunk0;
   __syncthreads();
+  int held = -1;  // the job whose laws are in shared memory
   for (int64_t gc = blockIdx.x; gc < total_chunks; gc += gridDim.x) {
-    const JobView& v = views[owner(starts, n_jobs, gc)];
+    const int job = n_jobs > 1 ? owner(starts, n_jobs, gc) : 0;
+    const JobView& v = views[job];
+    if (job != held) {  // (a block sum's barrier lies between the last use and this)
+      static_assert(sizeof(RayConst) % 4 == 0, "");
+      const int* src = reinterpret_cast<const int*>(v.ray);
+      int* dst = reinterpret_cast<int*>(law.ray);
+      for (int k = threadIdx.x; k < v.n_phases * (int)(sizeof(RayConst) / 4); k += blockDim.x) dst[k] = src[k];
+      if (threadIdx.x < kMaxPhases) law.kind[threadIdx.x] = v.kind[threadIdx.x];
+      held = job;
+      __syncthreads();
+    }
     const int64_t lc = gc - v.vchunk0;
     T acc[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 1
-    for (int sweep = 0; sweep < kVChunk / kMatBlock; ++sweep) {
-      const int64_t i = lc * kVChunk + sweep * kMatBlock + threadIdx.x;
+    for (int o = threadIdx.x; o < v.chunk; o += kMatBlock) {
+      const int64_t i = lc * v.chunk + o;
       if (i < v.nvox)
-        material_voxel<T, MODE>(i, v.nvox, v.phase, *v.tab, v.ray, (T)v.inv_n3, static_cast<const T*>(v.eps_raw),
+        material_voxel<T, MODE>(i, v.nvox, v.phase, *v.tab, law, (T)v.inv_n3, static_cast<const T*>(v.eps_raw),
                                 static_cast<const T*>(v.zn), static_cast<T*>(v.sig), static_cast<T*>(v.z), acc);
     }
     double accd[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) accd[c] = (double)acc[c];
-    block_sum_at<6>(accd, v.mat_part, v.n_vch, lc);
+    block_sum6_at(accd, v.mat_part, v.n_vch, lc);
   }
 }
 
@@ -381,35 +457,32 @@ __global__ void __launch_bounds__(kGamBlock) ms_gamma_batch_kernel(const JobView
   }
 }
 
-// Final sums of one problem's partials: warp c (c < 6) sums component c of
-// the material partials, warp 6 the error partials; lane l takes partials
-// l, l + 32, ... and the lanes combine in a fixed shuffle tree, so the order
-// depends only on the partial count (never on other problems in a batch).
-// Launch with kFinBlock threads.
-constexpr int kFinBlock = 224;
+// Final sums of one problem's partials (six stress components, the error) by
+// one block: each thread takes every blockDim-th partial of all seven, with
+// their loads in flight together, then the block's fixed shuffle tree.  The
+// order depends only on the partial counts and the block size (never on other
+// problems in a batch).  The 256^3 sums took 58 us with one warp a sum.
+constexpr int kFinBlock = 512;
 __device__ void finalize_sums(const double* __restrict__ mat_part, int n_mat, const double* __restrict__ gam_part,
                               int n_gam, double inv_n3, double floor_, Reduced* __restrict__ out) {
-  __shared__ double sh[7];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double s = 0.0;
-  if (w < 6) {
-    for (int b = lane; b < n_mat; b += 32) s += mat_part[w * n_mat + b];
-  } else if (w == 6) {
-    for (int b = lane; b < n_gam; b += 32) s += gam_part[b];
-  }
+  __shared__ double sum[7];
+  double a[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 4
+  for (int b = threadIdx.x; b < n_mat; b += blockDim.x)
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  if (lane == 0 && w < 7) sh[w] = s;
-  __syncthreads();
+    for (int c = 0; c < 6; ++c) a[c] += __ldcg(mat_part + (int64_t)c * n_mat + b);
+#pragma unroll 4
+  for (int b = threadIdx.x; b < n_gam; b += blockDim.x) a[6] += __ldcg(gam_part + b);
+  block_sum_at<7>(a, sum, 1, 0);
   if (threadIdx.x == 0) {
     double m[6];
-    for (int c = 0; c < 6; ++c) m[c] = sh[c] * inv_n3;
+    for (int c = 0; c < 6; ++c) m[c] = sum[c] * inv_n3;
     // sum |xi . c|^2 with xi = 2 pi k and c = sigma^ / N^3
-    const double num = sqrt(sh[6]) * kTwoPi * inv_n3;
+    const double num = sqrt(sum[6]) * kTwoPi * inv_n3;
     const double fro = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2] + 2.0 * (m[3] * m[3] + m[4] * m[4] + m[5] * m[5]));
     out->e = num / fmax(fro, floor_);
     for (int c = 0; c < 6; ++c) out->mean[c] = m[c];
-    out->res = sh[6];
+    out->res = sum[6];
   }
 }
 
@@ -420,24 +493,42 @@ __global__ void ms_finalize_kernel(const double* __restrict__ mat_part, int n_ma
 }
 
 // One block per job.
-__global__ void ms_finalize_batch_kernel(const JobView* __restrict__ views, Reduced* __restrict__ out) {
+__global__ void ms_finalize_batch_kernel(const JobView* __restrict__ views) {
   const JobView& v = views[blockIdx.x];
-  finalize_sums(v.mat_part, v.n_vch, v.gam_part, v.n_mch, v.inv_n3, v.mu0 * 1e-6, out + blockIdx.x);
+  finalize_sums(v.mat_part, v.n_vch, v.gam_part, v.n_mch, v.inv_n3, v.mu0 * 1e-6, v.red);
 }
 
 // Mean mode of the strain spectrum and of the inverse-transform input:
 // m = N^3 E (mixed boundary conditions move E during a load step).  One warp.
 template <class T>
 __global__ void ms_set_mean_kernel(typename cplx<T>::type* __restrict__ eps_hat, typename cplx<T>::type* __restrict__ sig_hat,
-                                   int64_t nmodes, double m0, double m1, double m2, double m3, double m4, double m5) {
-  const double m[6] = {m0, m1, m2, m3, m4, m5};
+                                   int64_t nmodes, double6 m) {
   const int q = threadIdx.x;
   if (q < 6) {
     typename cplx<T>::type v;
-    v.x = (T)m[q];
+    v.x = (T)m.v[q];
     v.y = T(0);
     eps_hat[q * nmodes] = v;
     sig_hat[q * nmodes] = v;
+  }
+}
+
+// The same for a spectrum whose inverse x pass is done (fft.cuh): the mean mode
+// is there a constant along x, which moves by d = N^3 dE; eps_hat's is set to m.
+template <class T>
+__global__ void ms_move_mean_kernel(typename cplx<T>::type* __restrict__ eps_hat, typename cplx<T>::type* __restrict__ sig_hat,
+                                    int N, double6 m, double6 d) {
+  const int Nh = N / 2 + 1;
+  const int64_t nmodes = (int64_t)N * N * Nh;
+  for (int i = threadIdx.x; i < 6 * N; i += blockDim.x) {
+    const int q = i / N, x = i % N;
+    sig_hat[q * nmodes + (int64_t)x * N * Nh].x += (T)d.v[q];
+    if (x == 0) {
+      typename cplx<T>::type v;
+      v.x = (T)m.v[q];
+      v.y = T(0);
+      eps_hat[q * nmodes] = v;
+    }
   }
 }
 

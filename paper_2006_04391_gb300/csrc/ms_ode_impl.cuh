@@ -99,9 +99,9 @@ __global__ void __launch_bounds__(kMatBlock) ms_material_ode_kernel(const JobVie
     const Ode23Ctl ctl{v.ode_rtol, v.ode_atol, v.ode_max};
     double acc[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 1
-    for (int sweep = 0; sweep < kVChunk / kMatBlock; ++sweep) {
-      const int64_t i = lc * kVChunk + sweep * kMatBlock + threadIdx.x;
-      material_voxel_ode<PAIR>(i, i < v.nvox, v, hs, ctl, acc);
+    for (int o = 0; o < v.chunk; o += kMatBlock) {
+      const int64_t i = lc * v.chunk + o + threadIdx.x;
+      material_voxel_ode<PAIR>(i, o + (int)threadIdx.x < v.chunk && i < v.nvox, v, hs, ctl, acc);
     }
     block_sum_at<6>(acc, v.mat_part, v.n_vch, lc);
   }

@@ -6,19 +6,21 @@
 // fields stay resident in HBM.  One iteration ("tick") of every active job:
 //
 //   material kernel   sigma, z = law(eps_raw / N^3, z_n)   + FP64 partial sums of sigma
-//   cuFFT R2C (x6)    sigma -> sig_hat                      (per job)
-//   gamma kernel      per mode: error partial sums (FP64), eps_hat -= Gamma0 : sig_hat,
-//                     and a copy of eps_hat into sig_hat's buffer for the inverse
-//   finalize kernel   fixed-order sums -> e and <sigma> (FP64) per job, one copy to host
-//   cuFFT C2R (x6)    eps_hat copy -> eps_raw (unnormalised: N^3 eps)   (per job)
+//   zy pass           sigma -> its (z, y) spectrum
+//   x + Green pass    x transform, per mode: error partial sums (FP64), eps_hat -= Gamma0 : sig_hat,
+//                     inverse x transform of the updated eps_hat; the job's last block sums the
+//                     partials in a fixed order -> e and <sigma> (FP64), written to host memory
+//   inverse zy pass   -> eps_raw (unnormalised: N^3 eps)
 //
-// The material, gamma and finalize kernels take every job of the tick in one
-// launch (ms_kernels.cuh); ms_run is a tick loop over a single job, the
-// serve_* API a tick loop over a job table with admission by an HBM budget.
-// The C2R output is never normalised in a separate pass: the material kernel
-// scales it by 1/N^3 as it loads it.  cuFFT may overwrite the input of a
-// multi-dimensional C2R, which is why the gamma kernel writes the updated
-// eps_hat twice (state and transform input).
+// The transforms are the library's own (fft.cuh) where the grid size has one,
+// one launch per pass for all jobs of a size; other sizes take cuFFT per job
+// around the batched Green kernel of ms_kernels.cuh.  ms_run is a tick loop
+// over a single job, the serve_* API a tick loop over a job table with
+// admission by an HBM budget.  The inverse transform's output is never
+// normalised in a separate pass: the material kernel scales it by 1/N^3 as it
+// loads it.  cuFFT may overwrite the input of a multi-dimensional C2R, which is
+// why its Green kernel writes the updated eps_hat twice (state and transform
+// input).
 #include <cufft.h>
 
 #include <algorithm>
@@ -29,10 +31,12 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <tuple>
 #include <vector>
 
 #include "adjoint_kernels.cuh"
 #include "common.cuh"
+#include "fft.h"
 #include "ms_kernels.cuh"
 #include "ms_ode.h"
 
@@ -59,17 +63,37 @@ template <class T> size_t field_bytes(int64_t nvox, int64_t nmodes) {
   return 4 * 6 * nvox * sizeof(T) + 2 * 6 * nmodes * sizeof(typename cplx<T>::type);
 }
 
-int64_t n_vchunks(int64_t nvox) { return (nvox + kVChunk - 1) / kVChunk; }
+// Voxels per chunk: at least eight chunks a SM before a chunk grows beyond one
+// warp's voxels (a 16^3 grid: 128 chunks of 32, not 4 of 1024; the law is a
+// chain of FP64 latencies, 383 -> 13 us there), whole blocks beyond one
+// block's.
+int chunk_of(int64_t nvox) {
+  const int64_t c = nvox / (8 * 152);
+  if (c < kMatBlock) return (int)std::max<int64_t>(32, (c + 31) / 32 * 32);
+  return (int)std::min<int64_t>(kVChunk, c / kMatBlock * kMatBlock);
+}
+int64_t n_vchunks(int64_t nvox) {
+  const int64_t c = chunk_of(nvox);
+  return (nvox + c - 1) / c;
+}
 int64_t n_mchunks(int64_t nmodes) { return (nmodes + kMChunk - 1) / kMChunk; }
+// Error partials of the Green pass, whichever of the two transforms a precision takes.
+int64_t n_gam_part(int N) {
+  int64_t n = n_mchunks((int64_t)N * N * (N / 2 + 1));
+  for (const FftOps* o : {fft_ops_f32(N), fft_ops_f64(N)})
+    if (o) n = std::max<int64_t>(n, o->green_tiles);
+  return n;
+}
 
 size_t job_bytes(int N, int precision) {
   const int64_t nv = (int64_t)N * N * N, nm = (int64_t)N * N * (N / 2 + 1);
   size_t b = field_bytes<double>(nv, nm) + (precision == MS_PREC_FP32_BULK ? field_bytes<float>(nv, nm) : 0);
-  b += (6 * n_vchunks(nv) + n_mchunks(nm)) * sizeof(double) + sizeof(PhaseTable) + (size_t)nv;  // + phase copy
+  b += (6 * n_vchunks(nv) + n_gam_part(N)) * sizeof(double) + sizeof(PhaseTable) + (size_t)nv;  // + phase copy
   return b;
 }
 
 size_t plan_bytes_one(int N, bool fp32) {
+  if (fp32 ? fft_ops_f32(N) : fft_ops_f64(N)) return (size_t)N * (fp32 ? sizeof(float2) : sizeof(double2));
   int n[3] = {N, N, N};
   const long long nv = (long long)N * N * N, nm = (long long)N * N * (N / 2 + 1);
   size_t total = 0, ws = 0;
@@ -88,18 +112,27 @@ size_t plan_bytes(int N, int precision) {
 
 // ------------------------------------------------------------------- engine
 
+// The transforms of one grid size and precision: the library's own kernels
+// (fft.cuh) with their twiddle table exp(-2 pi i m / N), or cuFFT plans.
 struct Plans {
+  const FftOps* ops = nullptr;
+  void* tw = nullptr;
   cufftHandle r2c = 0, c2r = 0;
 };
 
-// Stream, cuFFT plan cache and the per-tick job table shared by all jobs.
+// Stream, plan cache and the per-tick job table shared by all jobs.
 struct Engine {
   cudaStream_t stream = nullptr;
   std::map<std::pair<int, int>, Plans> plans;  // (N, fp32) -> plans
-  JobView* views_dev = nullptr;                // scratch: the tick's job table
-  JobView* views_host = nullptr;               // pinned staging
-  Reduced* red_dev = nullptr;
-  Reduced* red_host = nullptr;
+  // The tick's job table, twice: a job that goes on swaps its strain and stress
+  // buffers every tick, so ticks of the same jobs alternate between two tables
+  // and the table of two ticks ago is usually the one needed (no upload).
+  JobView* views_dev = nullptr;                // [2][cap]
+  JobView* views_host = nullptr;               // [2][cap] pinned: what views_dev holds
+  std::vector<JobView> views_new;
+  int views_n[2] = {0, 0}, views_slot = 0;
+  Reduced* red_host = nullptr;                 // [cap] page-locked: the kernels write each job's sums here
+  cudaEvent_t read = nullptr;                  // the tick's errors are in host memory
   int cap = 0;
   bool inited = false;
   int per_sm_mat[6] = {1, 1, 1, 1, 1, 1};  // FP64, FP32-fix, FP32 laws; ode23, ode12, ode23s laws
@@ -109,10 +142,10 @@ struct Engine {
     stream = s;
     cap = capacity;
     inited = true;
-    if (cudaMalloc((void**)&views_dev, cap * sizeof(JobView)) != cudaSuccess ||
-        cudaMallocHost((void**)&views_host, cap * sizeof(JobView)) != cudaSuccess ||
-        cudaMalloc((void**)&red_dev, cap * sizeof(Reduced)) != cudaSuccess ||
-        cudaMallocHost((void**)&red_host, cap * sizeof(Reduced)) != cudaSuccess) {
+    if (cudaMalloc((void**)&views_dev, 2 * cap * sizeof(JobView)) != cudaSuccess ||
+        cudaMallocHost((void**)&views_host, 2 * cap * sizeof(JobView)) != cudaSuccess ||
+        cudaMallocHost((void**)&red_host, cap * sizeof(Reduced)) != cudaSuccess ||
+        cudaEventCreateWithFlags(&read, cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
       return GSM_ENOMEM;
     }
@@ -139,6 +172,28 @@ struct Engine {
     auto it = plans.find(key);
     if (it == plans.end()) {
       Plans p;
+      p.ops = fp32 ? fft_ops_f32(N) : fft_ops_f64(N);
+      if (p.ops) {
+        std::vector<double2> tw(N);
+        for (int m = 0; m < N; ++m) {
+          const long double a = 2.0L * 3.141592653589793238462643383279502884L * m / N;
+          tw[m] = make_double2((double)std::cos(a), (double)-std::sin(a));
+        }
+        std::vector<float2> twf(N);
+        for (int m = 0; m < N; ++m) twf[m] = make_float2((float)tw[m].x, (float)tw[m].y);
+        const size_t bytes = N * (fp32 ? sizeof(float2) : sizeof(double2));
+        if (cudaMalloc(&p.tw, bytes) != cudaSuccess) {
+          cudaGetLastError();
+          return GSM_ENOMEM;
+        }
+        if (cudaMemcpy(p.tw, fp32 ? (const void*)twf.data() : (const void*)tw.data(), bytes, cudaMemcpyHostToDevice) !=
+            cudaSuccess) {
+          cudaFree(p.tw);
+          return GSM_ECUDA;
+        }
+        *out = &plans.emplace(key, p).first->second;
+        return GSM_OK;
+      }
       int n[3] = {N, N, N};
       const int nv = N * N * N, nm = N * N * (N / 2 + 1);
       if (cufftPlanMany(&p.r2c, 3, n, nullptr, 1, nv, nullptr, 1, nm, fp32 ? CUFFT_R2C : CUFFT_D2Z, 6) !=
@@ -160,12 +215,14 @@ struct Engine {
   ~Engine() {
     if (inited) cudaStreamSynchronize(stream);
     for (auto& kv : plans) {
+      cudaFree(kv.second.tw);
+      if (kv.second.ops) continue;
       cufftDestroy(kv.second.r2c);
       cufftDestroy(kv.second.c2r);
     }
+    if (read) cudaEventDestroy(read);
     cudaFree(views_dev);
     cudaFreeHost(views_host);
-    cudaFree(red_dev);
     cudaFreeHost(red_host);
   }
 };
@@ -192,6 +249,7 @@ struct Job {
   Fields<float> f32;
   double* mat_part = nullptr;
   double* gam_part = nullptr;
+  unsigned* arrived = nullptr;       // counter of the fused Green pass
   size_t bytes = 0;
   bool allocated = false;
   // load
@@ -214,6 +272,7 @@ struct Job {
   // state
   int step = 0, n_eval = 0, n32 = 0, since_best = 0;
   bool fp32_phase = false, need_start = true, done = false, notconv = false;
+  bool ahead = false;  // the next strain is being written into sig's buffer (tick)
   double best = 1e300;
   double E_prev[6] = {0, 0, 0, 0, 0, 0};  // macroscopic strain at the end of the previous step
   double E_cur[6] = {0, 0, 0, 0, 0, 0};   // macroscopic strain of the current iterate
@@ -291,6 +350,8 @@ void job_free(Job& j, cudaStream_t s) {
   free_fields(j.f32, s);
   if (j.mat_part) cudaFreeAsync(j.mat_part, s);
   if (j.gam_part) cudaFreeAsync(j.gam_part, s);
+  if (j.arrived) cudaFreeAsync(j.arrived, s);
+  j.arrived = nullptr;
   if (j.tab_dev) cudaFreeAsync(j.tab_dev, s);
   if (j.phase_owned) cudaFreeAsync(j.phase_owned, s);
   if (j.eps_prev) cudaFreeAsync(j.eps_prev, s);
@@ -309,7 +370,9 @@ int job_alloc(Job& j, cudaStream_t s, const uint8_t* phase_host) {
   bool ok = alloc_fields(j.f64, j.nvox, j.nmodes, s);
   if (ok && j.precision == MS_PREC_FP32_BULK) ok = alloc_fields(j.f32, j.nvox, j.nmodes, s);
   ok = ok && cudaMallocAsync((void**)&j.mat_part, 6 * (size_t)j.n_vch * sizeof(double), s) == cudaSuccess &&
-       cudaMallocAsync((void**)&j.gam_part, (size_t)j.n_mch * sizeof(double), s) == cudaSuccess &&
+       cudaMallocAsync((void**)&j.gam_part, (size_t)n_gam_part(j.N) * sizeof(double), s) == cudaSuccess &&
+       cudaMallocAsync((void**)&j.arrived, sizeof(unsigned), s) == cudaSuccess &&
+       cudaMemsetAsync(j.arrived, 0, sizeof(unsigned), s) == cudaSuccess &&
        cudaMallocAsync((void**)&j.tab_dev, sizeof(PhaseTable), s) == cudaSuccess;
   if (ok && phase_host) {
     ok = cudaMallocAsync((void**)&j.phase_owned, (size_t)j.nvox, s) == cudaSuccess &&
@@ -404,10 +467,28 @@ template <class T> Fields<T>& fields(Job& j);
 template <> Fields<double>& fields<double>(Job& j) { return j.f64; }
 template <> Fields<float>& fields<float>(Job& j) { return j.f32; }
 
-cufftResult exec_r2c(const Plans& p, double* in, cufftDoubleComplex* out) { return cufftExecD2Z(p.r2c, in, out); }
-cufftResult exec_r2c(const Plans& p, float* in, cufftComplex* out) { return cufftExecR2C(p.r2c, in, out); }
-cufftResult exec_c2r(const Plans& p, cufftDoubleComplex* in, double* out) { return cufftExecZ2D(p.c2r, in, out); }
-cufftResult exec_c2r(const Plans& p, cufftComplex* in, float* out) { return cufftExecC2R(p.c2r, in, out); }
+cufftResult lib_r2c(const Plans& p, double* in, cufftDoubleComplex* out) { return cufftExecD2Z(p.r2c, in, out); }
+cufftResult lib_r2c(const Plans& p, float* in, cufftComplex* out) { return cufftExecR2C(p.r2c, in, out); }
+cufftResult lib_c2r(const Plans& p, cufftDoubleComplex* in, double* out) { return cufftExecZ2D(p.c2r, in, out); }
+cufftResult lib_c2r(const Plans& p, cufftComplex* in, float* out) { return cufftExecC2R(p.c2r, in, out); }
+
+const JobList kNoList{};
+
+// Whole forward / inverse transform of one job's six components (the inverse
+// may overwrite its input; the library's own forward transform gives twice the
+// spectrum, fft.cuh).
+template <class T, class C> bool exec_r2c(const Plans& p, T* in, C* out, cudaStream_t s) {
+  if (!p.ops) return lib_r2c(p, in, out) == CUFFT_SUCCESS;
+  p.ops->zy_fwd(nullptr, kNoList, 1, in, out, p.tw, s);
+  p.ops->x_fwd(nullptr, kNoList, 1, out, p.tw, s);
+  return true;
+}
+template <class T, class C> bool exec_c2r(const Plans& p, C* in, T* out, cudaStream_t s) {
+  if (!p.ops) return lib_c2r(p, in, out) == CUFFT_SUCCESS;
+  p.ops->x_inv(nullptr, kNoList, 1, in, p.tw, s);
+  p.ops->zy_inv(nullptr, kNoList, 1, in, out, p.tw, s);
+  return true;
+}
 
 int elt_grid(int64_t n) { return grid_cap(n, 256, 8); }
 
@@ -427,19 +508,28 @@ template <class T> int spectrum_start(Engine& g, Job& j, const double* E, const 
   for (int q = 0; q < 6; ++q) d[q] = n3 * (E[q] - E_prev[q]);
   ms_add_uniform_kernel<T><<<elt_grid(j.nvox), 256, 0, g.stream>>>(j.nvox, f.eps_raw, d[0], d[1], d[2], d[3], d[4],
                                                                      d[5]);
-  if (exec_r2c(*p, f.eps_raw, f.sig_hat) != CUFFT_SUCCESS) return GSM_ECUDA;
-  ms_spectrum_init_kernel<T><<<elt_grid(j.nmodes), 256, 0, g.stream>>>(j.nmodes, f.sig_hat, f.eps_hat, 1.0 / n3, n3,
+  if (!exec_r2c(*p, f.eps_raw, f.sig_hat, g.stream)) return GSM_ECUDA;
+  ms_spectrum_init_kernel<T><<<elt_grid(j.nmodes), 256, 0, g.stream>>>(j.nmodes, f.sig_hat, f.eps_hat, (p->ops ? 0.5 : 1.0) / n3, n3,
                                                                          E[0], E[1], E[2], E[3], E[4], E[5]);
   count_launch(2);
   return cudaGetLastError() == cudaSuccess ? GSM_OK : GSM_ECUDA;
 }
 
+// The strain of the next evaluation, from the spectrum the Green pass left in
+// sig_hat.
 template <class T> int inverse(Engine& g, Job& j) {
   Fields<T>& f = fields<T>(j);
+  if (j.ahead) {  // already queued by the tick, into sig's buffer
+    std::swap(f.eps_raw, f.sig);
+    j.ahead = false;
+    return GSM_OK;
+  }
   Plans* p = nullptr;
   int rc = g.get_plans(j.N, sizeof(T) == 4, &p);
   if (rc != GSM_OK) return rc;
-  return exec_c2r(*p, f.sig_hat, f.eps_raw) == CUFFT_SUCCESS ? GSM_OK : GSM_ECUDA;
+  if (!p->ops) return lib_c2r(*p, f.sig_hat, f.eps_raw) == CUFFT_SUCCESS ? GSM_OK : GSM_ECUDA;
+  p->ops->zy_inv(nullptr, kNoList, 1, f.sig_hat, f.eps_raw, p->tw, g.stream);
+  return GSM_OK;
 }
 
 int cap_of(const Job& j) { return j.forced.empty() ? j.max_iter : j.forced[j.step]; }
@@ -549,17 +639,24 @@ int step_start(Engine& g, Job& j) {
 // Mixed boundary conditions: dE_s = (C0_ss)^-1 (Sigma_s - <sigma>_s) on the
 // prescribed-stress components, written into the mean mode of the strain
 // spectrum and of the inverse-transform input.
-template <class T> void move_mean(Engine& g, Job& j, const double (&dS)[6]) {
+template <class T> int move_mean(Engine& g, Job& j, const double (&dS)[6]) {
+  const double n3 = (double)j.nvox;
+  double6 m{}, dm{};
   for (int a = 0; a < j.n_s; ++a) {
     double d = 0.0;
     for (int b = 0; b < j.n_s; ++b) d += j.C0ss_inv[a * j.n_s + b] * dS[j.s_idx[b]];
     j.E_cur[j.s_idx[a]] += d;
+    dm.v[j.s_idx[a]] = n3 * d;
   }
-  const double n3 = (double)j.nvox;
+  for (int q = 0; q < 6; ++q) m.v[q] = n3 * j.E_cur[q];
   Fields<T>& f = fields<T>(j);
-  ms_set_mean_kernel<T><<<1, 32, 0, g.stream>>>(f.eps_hat, f.sig_hat, j.nmodes, n3 * j.E_cur[0], n3 * j.E_cur[1],
-                                                n3 * j.E_cur[2], n3 * j.E_cur[3], n3 * j.E_cur[4], n3 * j.E_cur[5]);
+  Plans* p = nullptr;
+  const int rc = g.get_plans(j.N, sizeof(T) == 4, &p);
+  if (rc != GSM_OK) return rc;
+  if (p->ops) ms_move_mean_kernel<T><<<1, 256, 0, g.stream>>>(f.eps_hat, f.sig_hat, j.N, m, dm);
+  else ms_set_mean_kernel<T><<<1, 32, 0, g.stream>>>(f.eps_hat, f.sig_hat, j.nmodes, m);
   count_launch();
+  return GSM_OK;
 }
 
 // FP32 -> FP64 hand-over within a step: the FP32 strain of the last
@@ -572,7 +669,10 @@ int switch_to_fp64(Engine& g, Job& j) {
   cudaMemcpyAsync(j.f64.sig_hat, j.f64.eps_hat, 6 * j.nmodes * sizeof(cufftDoubleComplex), cudaMemcpyDeviceToDevice,
                   g.stream);
   j.fp32_phase = false;
-  return inverse<double>(g, j);
+  Plans* p = nullptr;
+  rc = g.get_plans(j.N, false, &p);
+  if (rc != GSM_OK) return rc;
+  return exec_c2r(*p, j.f64.sig_hat, j.f64.eps_raw, g.stream) ? GSM_OK : GSM_ECUDA;
 }
 
 // After the tick's evaluation: convergence, precision switch, step end.
@@ -604,7 +704,10 @@ int post_eval(Engine& g, Job& j, const Reduced& r) {
       ++j.since_best;
     }
     if (e < std::max(j.switch_tol, j.tol) || j.since_best >= 20 || j.n_eval >= cap - 1) return switch_to_fp64(g, j);
-    if (j.stress_mask) move_mean<float>(g, j, dS);
+    if (j.stress_mask) {
+      const int rc = move_mean<float>(g, j, dS);
+      if (rc != GSM_OK) return rc;
+    }
     return inverse<float>(g, j);
   }
   bool end = false, conv = false;
@@ -616,7 +719,10 @@ int post_eval(Engine& g, Job& j, const Reduced& r) {
     end = true;
   }
   if (!end) {
-    if (j.stress_mask) move_mean<double>(g, j, dS);
+    if (j.stress_mask) {
+      const int rc = move_mean<double>(g, j, dS);
+      if (rc != GSM_OK) return rc;
+    }
     return inverse<double>(g, j);
   }
   if (!conv) j.notconv = true;
@@ -655,6 +761,7 @@ int tick(Engine& g, const std::vector<Job*>& jobs) {
       if (rc != GSM_OK) return rc;
       j->need_start = false;
     }
+  for (Job* j : jobs) j->ahead = false;
   // launch groups: FP64 fields + FP64 laws, FP64 fields + FP32-fix laws,
   // FP64 fields + ode23 / ode12 / ode23s laws, FP32 fields (FP64 groups
   // first: one Green launch)
@@ -664,21 +771,28 @@ int tick(Engine& g, const std::vector<Job*>& jobs) {
     if (j->integrator >= 1) return 1 + j->integrator;
     return j->law_mode == MODE_FP32_FIX ? 1 : 0;
   };
-  std::vector<Job*> order;
-  order.reserve(n);
+  std::vector<Job*> order(jobs.begin(), jobs.end());
+  std::vector<Plans*> plan(n);
+  auto own = [](const Job* j) { return (j->fp32_phase ? fft_ops_f32(j->N) : fft_ops_f64(j->N)) != nullptr; };
+  // by launch group, the library's own transforms first, by grid size
+  std::stable_sort(order.begin(), order.end(), [&](const Job* a, const Job* b) {
+    return std::make_tuple(key(a), own(a) ? 0 : 1, a->N) < std::make_tuple(key(b), own(b) ? 0 : 1, b->N);
+  });
   int gstart[kGroups + 1] = {0, 0, 0, 0, 0, 0, 0};
-  for (int k = 0; k < kGroups; ++k) {
-    for (Job* j : jobs)
-      if (key(j) == k) order.push_back(j);
-    gstart[k + 1] = (int)order.size();
+  for (int i = 0; i < n; ++i) {
+    const int rc = g.get_plans(order[i]->N, order[i]->fp32_phase, &plan[i]);
+    if (rc != GSM_OK) return rc;
+    ++gstart[key(order[i]) + 1];
   }
-  int64_t vtot[kGroups] = {0, 0, 0, 0, 0, 0}, mtot[2] = {0, 0};
+  for (int k = 0; k < kGroups; ++k) gstart[k + 1] += gstart[k];
+  int64_t vtot[kGroups] = {0, 0, 0, 0, 0, 0}, mtot[kGroups] = {0, 0, 0, 0, 0, 0};
+  g.views_new.resize(n);
   for (int i = 0; i < n; ++i) {
     Job& j = *order[i];
     const int k = key(&j);
-    const int pk = k == kF32 ? 1 : 0;
     const bool f = j.fp32_phase;
-    JobView& v = g.views_host[i];
+    JobView& v = g.views_new[i];
+    std::memset(&v, 0, sizeof v);
     v.phase = j.phase;
     v.eps_raw = f ? (const void*)j.f32.eps_raw : (const void*)j.f64.eps_raw;
     v.zn = f ? (const void*)j.f32.zn : (const void*)j.f64.zn;
@@ -686,84 +800,129 @@ int tick(Engine& g, const std::vector<Job*>& jobs) {
     v.z = f ? (void*)j.f32.z : (void*)j.f64.z;
     v.sig_hat = f ? (void*)j.f32.sig_hat : (void*)j.f64.sig_hat;
     v.eps_hat = f ? (void*)j.f32.eps_hat : (void*)j.f64.eps_hat;
+    v.eps_out = v.sig;  // (the stress is not needed once its spectrum is formed)
     v.mat_part = j.mat_part;
     v.gam_part = j.gam_part;
+    v.red = g.red_host + i;
+    v.arrived = plan[i]->ops ? j.arrived : nullptr;
     v.tab = j.tab_dev;
     v.nvox = j.nvox;
     v.nmodes = j.nmodes;
     v.vchunk0 = vtot[k];
-    v.mchunk0 = mtot[pk];
+    v.mchunk0 = mtot[k];
     v.n_vch = j.n_vch;
-    v.n_mch = j.n_mch;
+    v.n_mch = plan[i]->ops ? plan[i]->ops->green_tiles : j.n_mch;
+    v.chunk = chunk_of(j.nvox);
     v.N = j.N;
-    v.pad1 = 0;
+    v.n_phases = j.n_phases;
     std::memcpy(v.ray, j.ray, j.n_phases * sizeof(RayConst));
+    std::memcpy(v.kind, j.tab_host.kind, sizeof(v.kind));
     v.h = j.h[j.step];
     v.inv_h = 1.0 / v.h;
     v.inv_n3 = 1.0 / (double)j.nvox;
-    v.lam0 = j.lam0;
-    v.mu0 = j.mu0;
+    set_reference(v, j.lam0, j.mu0);
     v.eps_prev = j.eps_prev;
     v.alpha_n = j.alpha_n;
     v.alpha = j.alpha;
     v.ode_rtol = j.ode_rtol;
     v.ode_atol = j.ode_atol;
     v.ode_max = j.ode_max;
-    v.pad2 = 0;
     vtot[k] += j.n_vch;
-    mtot[pk] += j.n_mch;
+    if (!plan[i]->ops) mtot[k] += j.n_mch;
   }
   cudaStream_t s = g.stream;
-  cudaMemcpyAsync(g.views_dev, g.views_host, n * sizeof(JobView), cudaMemcpyHostToDevice, s);
+  g.views_slot ^= 1;
+  JobView* const views = g.views_dev + g.views_slot * g.cap;
+  JobView* const staged = g.views_host + g.views_slot * g.cap;
+  // (the slot's previous upload, two ticks ago, has completed)
+  if (g.views_n[g.views_slot] != n || std::memcmp(staged, g.views_new.data(), n * sizeof(JobView)) != 0) {
+    std::memcpy(staged, g.views_new.data(), n * sizeof(JobView));
+    g.views_n[g.views_slot] = n;
+    cudaMemcpyAsync(views, staged, n * sizeof(JobView), cudaMemcpyHostToDevice, s);
+  }
   const int64_t sms = sm_count();
   if (gstart[1] > gstart[0]) {
     const int grid = (int)std::min<int64_t>(vtot[0], sms * g.per_sm_mat[0]);
-    ms_material_batch_kernel<double, MODE_FP64><<<grid, kMatBlock, 0, s>>>(g.views_dev + gstart[0],
+    ms_material_batch_kernel<double, MODE_FP64><<<grid, kMatBlock, 0, s>>>(views + gstart[0],
                                                                           gstart[1] - gstart[0], vtot[0]);
     count_launch();
   }
   if (gstart[2] > gstart[1]) {
     const int grid = (int)std::min<int64_t>(vtot[1], sms * g.per_sm_mat[1]);
-    ms_material_batch_kernel<double, MODE_FP32_FIX><<<grid, kMatBlock, 0, s>>>(g.views_dev + gstart[1],
+    ms_material_batch_kernel<double, MODE_FP32_FIX><<<grid, kMatBlock, 0, s>>>(views + gstart[1],
                                                                               gstart[2] - gstart[1], vtot[1]);
     count_launch();
   }
   for (int k = 2; k <= 4; ++k)
     if (gstart[k + 1] > gstart[k]) {
       const int grid = (int)std::min<int64_t>(vtot[k], sms * g.per_sm_mat[k + 1]);
-      ms_launch_material_ode(k - 2, grid, s, g.views_dev + gstart[k], gstart[k + 1] - gstart[k], vtot[k]);
+      ms_launch_material_ode(k - 2, grid, s, views + gstart[k], gstart[k + 1] - gstart[k], vtot[k]);
       count_launch();
     }
   if (gstart[kF32 + 1] > gstart[kF32]) {
     const int grid = (int)std::min<int64_t>(vtot[kF32], sms * g.per_sm_mat[2]);
-    ms_material_batch_kernel<float, MODE_FP32><<<grid, kMatBlock, 0, s>>>(g.views_dev + gstart[kF32],
+    ms_material_batch_kernel<float, MODE_FP32><<<grid, kMatBlock, 0, s>>>(views + gstart[kF32],
                                                                          gstart[kF32 + 1] - gstart[kF32], vtot[kF32]);
     count_launch();
   }
-  for (Job* j : order) {
-    Plans* p = nullptr;
-    int rc = g.get_plans(j->N, j->fp32_phase, &p);
-    if (rc != GSM_OK) return rc;
-    const cufftResult fr =
-        j->fp32_phase ? exec_r2c(*p, j->f32.sig, j->f32.sig_hat) : exec_r2c(*p, j->f64.sig, j->f64.sig_hat);
-    if (fr != CUFFT_SUCCESS) return GSM_ECUDA;
+  // forward transforms and the Green update: one launch per pass for all jobs
+  // of one grid size and precision, or cuFFT per job and the batched kernel
+  auto run_end = [&](int i) {
+    int e = i + 1;
+    while (e < n && plan[e] == plan[i]) ++e;
+    return e;
+  };
+  for (int i = 0; i < n;) {
+    const Plans& p = *plan[i];
+    if (!p.ops) {
+      Job* j = order[i++];
+      const cufftResult fr =
+          j->fp32_phase ? lib_r2c(p, j->f32.sig, j->f32.sig_hat) : lib_r2c(p, j->f64.sig, j->f64.sig_hat);
+      if (fr != CUFFT_SUCCESS) return GSM_ECUDA;
+      continue;
+    }
+    const int e = run_end(i);
+    JobList list;
+    for (int q = i; q < e; ++q) list.at[q - i] = (uint8_t)q;
+    p.ops->zy_fwd(views, list, e - i, nullptr, nullptr, p.tw, s);
+    p.ops->x_green(views, list, e - i, p.tw, s);
+    i = e;
   }
-  if (gstart[kF32] > gstart[0]) {
-    const int grid = (int)std::min<int64_t>(mtot[0], sms * g.per_sm_gam[0]);
-    ms_gamma_batch_kernel<double><<<grid, kGamBlock, 0, s>>>(g.views_dev + gstart[0], gstart[kF32] - gstart[0],
-                                                             mtot[0]);
-    count_launch();
+  for (int k = 0; k < kGroups; ++k) {
+    if (mtot[k] == 0) continue;
+    int i0 = gstart[k];
+    while (plan[i0]->ops) ++i0;
+    const int cnt = gstart[k + 1] - i0, f = k == kF32 ? 1 : 0;
+    const int grid = (int)std::min<int64_t>(mtot[k], sms * g.per_sm_gam[f]);
+    if (f) ms_gamma_batch_kernel<float><<<grid, kGamBlock, 0, s>>>(views + i0, cnt, mtot[k]);
+    else ms_gamma_batch_kernel<double><<<grid, kGamBlock, 0, s>>>(views + i0, cnt, mtot[k]);
+    ms_finalize_batch_kernel<<<cnt, kFinBlock, 0, s>>>(views + i0);
+    count_launch(2);
   }
-  if (gstart[kF32 + 1] > gstart[kF32]) {
-    const int grid = (int)std::min<int64_t>(mtot[1], sms * g.per_sm_gam[1]);
-    ms_gamma_batch_kernel<float><<<grid, kGamBlock, 0, s>>>(g.views_dev + gstart[kF32],
-                                                            gstart[kF32 + 1] - gstart[kF32], mtot[1]);
-    count_launch();
+  if (cudaEventRecord(g.read, s) != cudaSuccess) return GSM_ECUDA;
+  // While the errors travel to the host, the next strain is formed in the
+  // buffer of the stress, which is not needed any more; a job that goes on
+  // swaps the two, one whose step ends here keeps the strain of this
+  // evaluation.  (Not where the step is known to end, nor where the host still
+  // moves the mean strain.)
+  for (int i = 0; i < n;) {
+    const Plans& p = *plan[i];
+    const int e = run_end(i);
+    JobList list;
+    int cnt = 0;
+    for (int q = i; p.ops && q < e; ++q) {
+      Job& j = *order[q];
+      const int last = cap_of(j) - (j.fp32_phase ? 1 : 0);
+      if (j.stress_mask || j.n_eval + 1 >= last) continue;
+      j.ahead = true;
+      list.at[cnt++] = (uint8_t)q;
+    }
+    if (cnt) {
+      p.ops->zy_inv(views, list, cnt, nullptr, nullptr, p.tw, s);
+    }
+    i = e;
   }
-  ms_finalize_batch_kernel<<<n, kFinBlock, 0, s>>>(g.views_dev, g.red_dev);
-  count_launch();
-  cudaMemcpyAsync(g.red_host, g.red_dev, n * sizeof(Reduced), cudaMemcpyDeviceToHost, s);
-  if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return GSM_ECUDA;
+  if (cudaEventSynchronize(g.read) != cudaSuccess || cudaGetLastError() != cudaSuccess) return GSM_ECUDA;
   for (int i = 0; i < n; ++i) {
     int rc = post_eval(g, *order[i], g.red_host[i]);
     if (rc != GSM_OK) return rc;
@@ -1195,22 +1354,30 @@ int ms_adjoint(ms_tape_handle th, const double* w, int phase_id, double tol, int
     // normalised in the tape's CG arrays, C_t p in sig, G (.) through sig_hat /
     // eps_hat into eps_raw as -N^3 G (.)
     JobView& v = g.views_host[0];
+    g.views_n[0] = 0;  // (the tick's table in this slot is overwritten)
     std::memset(&v, 0, sizeof v);
     v.sig_hat = j.f64.sig_hat;
     v.eps_hat = j.f64.eps_hat;
     v.mat_part = j.mat_part;
     v.gam_part = j.gam_part;
+    v.red = g.red_host;
     v.nvox = nv;
     v.nmodes = j.nmodes;
     v.n_vch = 0;
-    v.n_mch = j.n_mch;
+    v.n_mch = pl->ops ? pl->ops->green_tiles : j.n_mch;
+    v.project = 1;
     v.N = j.N;
     v.inv_n3 = inv_n3;
-    v.lam0 = 0.0;
-    v.mu0 = 0.5;
+    set_reference(v, 0.0, 0.5);
     cudaMemcpyAsync(g.views_dev, g.views_host, sizeof(JobView), cudaMemcpyHostToDevice, s);
     const int gam_grid = (int)std::min<int64_t>(j.n_mch, (int64_t)sm_count() * g.per_sm_gam[0]);
     auto apply_G = [&](const double* tau) -> int {
+      if (pl->ops) {
+        pl->ops->zy_fwd(nullptr, kNoList, 1, tau, j.f64.sig_hat, pl->tw, s);
+        pl->ops->x_green(g.views_dev, kNoList, 1, pl->tw, s);
+        pl->ops->zy_inv(nullptr, kNoList, 1, j.f64.sig_hat, j.f64.eps_raw, pl->tw, s);
+        return GSM_OK;
+      }
       if (cufftExecD2Z(pl->r2c, const_cast<double*>(tau), j.f64.sig_hat) != CUFFT_SUCCESS) return GSM_ECUDA;
       cudaMemsetAsync(j.f64.eps_hat, 0, 6 * j.nmodes * sizeof(cufftDoubleComplex), s);
       ms_gamma_batch_kernel<double><<<gam_grid, kGamBlock, 0, s>>>(g.views_dev, 1, j.n_mch);
@@ -1307,23 +1474,27 @@ int ms_adjoint(ms_tape_handle th, const double* w, int phase_id, double tol, int
       v.eps_hat = j.f64.eps_hat;
       v.mat_part = j.mat_part;
       v.gam_part = j.gam_part;
+      v.red = g.red_host;
       v.nvox = nv;
       v.nmodes = j.nmodes;
       v.n_vch = 0;
-      v.n_mch = j.n_mch;
+      v.n_mch = pl->ops ? pl->ops->green_tiles : j.n_mch;
       v.N = j.N;
       v.inv_n3 = inv_n3;
-      v.lam0 = lam0;
-      v.mu0 = mu0;
+      set_reference(v, lam0, mu0);
       cudaMemcpyAsync(g.views_dev, g.views_host, sizeof(JobView), cudaMemcpyHostToDevice, s);
       double first = -1.0;
       for (; it < max_iter; ++it) {
         adj_tau_kernel<<<elt_grid(nv), 256, 0, s>>>(nv, t.Ct21, t.a_u, j.f64.eps_raw, inv_n3, j.f64.sig);
-        if (cufftExecD2Z(pl->r2c, j.f64.sig, j.f64.sig_hat) != CUFFT_SUCCESS) return GSM_ECUDA;
-        ms_gamma_batch_kernel<double><<<gam_grid, kGamBlock, 0, s>>>(g.views_dev, 1, j.n_mch);
-        ms_finalize_batch_kernel<<<1, kFinBlock, 0, s>>>(g.views_dev, g.red_dev);
+        if (pl->ops) {
+          pl->ops->zy_fwd(nullptr, kNoList, 1, j.f64.sig, j.f64.sig_hat, pl->tw, s);
+          pl->ops->x_green(g.views_dev, kNoList, 1, pl->tw, s);
+        } else {
+          if (cufftExecD2Z(pl->r2c, j.f64.sig, j.f64.sig_hat) != CUFFT_SUCCESS) return GSM_ECUDA;
+          ms_gamma_batch_kernel<double><<<gam_grid, kGamBlock, 0, s>>>(g.views_dev, 1, j.n_mch);
+        }
+        ms_finalize_batch_kernel<<<1, kFinBlock, 0, s>>>(g.views_dev);
         count_launch(3);
-        cudaMemcpyAsync(g.red_host, g.red_dev, sizeof(Reduced), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) return GSM_ECUDA;
         const double r = std::sqrt(g.red_host->res);
         if (first < 0.0) first = r;
@@ -1331,7 +1502,11 @@ int ms_adjoint(ms_tape_handle th, const double* w, int phase_id, double tol, int
           conv = true;
           break;
         }
-        if (cufftExecZ2D(pl->c2r, j.f64.sig_hat, j.f64.eps_raw) != CUFFT_SUCCESS) return GSM_ECUDA;
+        if (pl->ops) {
+          pl->ops->zy_inv(nullptr, kNoList, 1, j.f64.sig_hat, j.f64.eps_raw, pl->tw, s);
+        } else if (cufftExecZ2D(pl->c2r, j.f64.sig_hat, j.f64.eps_raw) != CUFFT_SUCCESS) {
+          return GSM_ECUDA;
+        }
       }
       if (conv) ++it;  // the evaluation that met the tolerance
     }
