@@ -31,6 +31,7 @@ template <class T> struct LawParams {
   T b_Psi;
   T H_kin;        // kinematic hardening modulus H (MichelSuquet)
   T sig_Y;        // yield stress, K(alpha) = sigma_Y (MichelSuquet)
+  T L_ode;        // flow factor 6 mu c_Psi b_Psi (12 mu^2)^(b_Psi - 1) (NortonDev, ode_ray.cuh)
 };
 
 // Linear elasticity: psi = 1/2 eps^T C eps, no internal variables.
@@ -155,6 +156,7 @@ struct NortonDev {
 // law is integrated in its force-potential form only (gsm_update_ode23).
 struct MichelSuquet {
   static constexpr int NY = 6;
+  static constexpr bool kRay = false;
 
   template <class EP, class YP, class P> AD_HD static auto psi(const EP& e, const YP& y, const P& p) {
     using ad::get;

@@ -45,7 +45,7 @@ __device__ __forceinline__ void material_voxel_ode(int64_t i, bool in, const Job
     double zi[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) zi[c] = nor ? __ldg(zn + c * nvox + i) : 0.0;
-    if (nor) w.init(p, e0, e, zi, hs.h);
+    if (nor) w.init(p, e0, e, zi, hs);
     else w.done = true;
     for (;;) {
       if (all_done(w.done)) break;
@@ -65,7 +65,7 @@ __device__ __forceinline__ void material_voxel_ode(int64_t i, bool in, const Job
 #pragma unroll
     for (int c = 0; c < 6; ++c) zi[c] = kin ? __ldg(zn + c * nvox + i) : 0.0;
     zi[6] = kin ? __ldg(v.alpha_n + i) : 0.0;
-    if (kin) w.init(p, e0, e, zi, hs.h);
+    if (kin) w.init(p, e0, e, zi, hs);
     else w.done = true;
     for (;;) {
       if (all_done(w.done)) break;

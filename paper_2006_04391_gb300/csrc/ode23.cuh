@@ -303,7 +303,7 @@ template <class Law, bool TAN, int PAIR = ERK_BS23> struct ErkVoxel {
   // zn: the NZ stored internal variables (z in Voigt order, then alpha, ...);
   // B: the law's blocks (psi_const_blocks), required with TAN
   AD_HD void init(const LawParams<double>& p, const double (&e0)[6], const double (&e1)[6], const double (&zn)[NZ],
-                  double h, const PsiBlocks<NY>* B = nullptr) {
+                  const Step& hs, const PsiBlocks<NY>* B = nullptr) {
     blk = B;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
@@ -326,7 +326,7 @@ template <class Law, bool TAN, int PAIR = ERK_BS23> struct ErkVoxel {
     ode_rhs<Law, TAN>(p, epsn, de, 0.0, s, k1, K1, blk);
     ode_stress<Law, TAN>(p, epsn, de, 0.0, s, sig_old, C_old, blk);
     t = 0.0;
-    dt = h;
+    dt = hs.h;
     n_acc = n_rej = 0;
     flags = 0;
     last_rejected = false;
@@ -854,7 +854,7 @@ template <class Law, bool TAN> struct RosVoxel {
   }
 
   AD_HD void init(const LawParams<double>& p, const double (&e0)[6], const double (&e1)[6], const double (&zn)[NZ],
-                  double h, const PsiBlocks<NY>* B = nullptr) {
+                  const Step& hs, const PsiBlocks<NY>* B = nullptr) {
     blk = B;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
@@ -876,9 +876,9 @@ template <class Law, bool TAN> struct RosVoxel {
     }
     ode_rhs<Law, TAN>(p, epsn, de, 0.0, s, F0, G0, blk);
     ode_stress<Law, TAN>(p, epsn, de, 0.0, s, sig_old, C_old, blk);
-    refresh(p, 0.0, 1.0 / h);
+    refresh(p, 0.0, 1.0 / hs.h);
     t = 0.0;
-    dt = h;
+    dt = hs.h;
     n_acc = n_rej = 0;
     flags = 0;
     last_rejected = false;
@@ -1100,9 +1100,23 @@ template <class Law, bool TAN> struct RosVoxel {
   }
 };
 
-// The voxel state of integrator PAIR.
+}  // namespace gsm
+
+#include "ode_ray.cuh"
+
+namespace gsm {
+
+// The voxel state of integrator PAIR (an explicit pair of a proportional law
+// without tangent: ode_ray.cuh).
+template <class Law, bool TAN, int PAIR> struct OdeVoxelOf {
+  using type = ErkVoxel<Law, TAN, PAIR>;
+};
+template <class Law, bool TAN> struct OdeVoxelOf<Law, TAN, ROS_23S> {
+  using type = RosVoxel<Law, TAN>;
+};
 template <class Law, bool TAN, int PAIR>
-using OdeVoxel = std::conditional_t<PAIR == ROS_23S, RosVoxel<Law, TAN>, ErkVoxel<Law, TAN, PAIR == ROS_23S ? 0 : PAIR>>;
+using OdeVoxel = std::conditional_t<Law::kRay && !TAN && PAIR != ROS_23S, RayErkVoxel<Law, PAIR>,
+                                    typename OdeVoxelOf<Law, TAN, PAIR>::type>;
 
 // One voxel, start to end (single thread; the kernel schedules ErkVoxel
 // states per lane itself).
@@ -1114,11 +1128,11 @@ AD_HD unsigned voxel_ode23(const LawParams<double>& p, const double (&epsn)[6], 
   if constexpr (TAN) {
     PsiBlocks<Law::NY> B;
     psi_const_blocks<Law>(p, B);
-    v.init(p, epsn, eps1, zn, hs.h, &B);
+    v.init(p, epsn, eps1, zn, hs, &B);
     while (!v.done) v.attempt(p, hs, ctl);
     return v.finish(hs.h, sig, z, C36);
   } else {
-    v.init(p, epsn, eps1, zn, hs.h);
+    v.init(p, epsn, eps1, zn, hs);
     while (!v.done) v.attempt(p, hs, ctl);
     return v.finish(hs.h, sig, z, C36);
   }

@@ -1,0 +1,209 @@
+// The explicit pairs (ode23, ode12) for a proportional law without tangent, in
+// its elastic deviatoric strain.
+//
+// With psi isotropic and Psi = c_Psi (s_A^2)^b_Psi, s_A the von Mises norm of
+// A = -psi_y, the flow is ydot = Lambda x with x the y-components of
+// dev(eps) - P y and
+//   Lambda = 6 mu c_Psi b_Psi (12 mu^2 Q)^(b_Psi - 1) = L_ode Q^(b_Psi - 1),
+//   Q = x0^2 + x1^2 + x0 x1 + (x2^2 + x3^2 + x4^2)/4     (s_A^2 = 12 mu^2 Q).
+// The strain is linear over the step, so x obeys the autonomous equation
+//   xdot = edot - Lambda(x) x,
+// and a Runge-Kutta method applied to x is the one applied to y (affine
+// change of variable; the stage abscissae equal the row sums).  The stresses
+// are sigma = kappa tr(eps) 1 + 2 mu x, and the pair's stress difference is
+// 2 mu times the embedded difference of x: no stress is evaluated twice and
+// the difference does not cancel.
+//
+// Bound: the FP64 pipe.  The AD sweeps of ode23.cuh took about 800 FP64
+// operations an attempt; this takes about 200 (odd integer n: Q^(b_Psi - 1) is
+// a product of Q) or 290 (else: the table power).  Measured on 200 k voxels, n =
+// 5, rtol 1e-3: 7568 -> 3502 us.
+#pragma once
+
+// (included by ode23.cuh)
+
+namespace gsm {
+
+// |a| > |b| ? |a| : |b| on the integer pipe (a NaN wins).
+AD_HD double absmax_bits(double a, double b) {
+  const uint64_t m = 0x7fffffffffffffffull;
+  const uint64_t x = fpow::bits_of(a) & m, y = fpow::bits_of(b) & m;
+  return fpow::double_of(x > y ? x : y);
+}
+
+template <class Law, int PAIR> struct RayErkVoxel {
+  double x[5], k1[5], ed[5];  // elastic deviatoric strain, its rate, the strain rate
+  double e0[5], de[5];        // y-components of dev(eps_n) and of dev(eps_{n+1}) - dev(eps_n)
+  double hyd0, dhyd;          // kappa tr(eps_n) and its increment
+  double sig_old[6];
+  double t, dt;
+  int n_acc, n_rej;
+  unsigned flags;
+  bool last_rejected, done;
+
+  AD_HD static double lambda(const LawParams<double>& p, const double (&v)[5]) {
+    const double Q = fma(v[0], v[0] + v[1], v[1] * v[1]) + 0.25 * fma(v[4], v[4], fma(v[3], v[3], v[2] * v[2]));
+    // b_Psi - 1 a small integer, from the bits (the same for every lane; an FP64
+    // compare or conversion would occupy the FP64 pipe)
+    const uint64_t b = fpow::bits_of(p.b_Psi);
+    if (b == fpow::bits_of(3.0)) return p.L_ode * (Q * Q);
+    if (b == fpow::bits_of(2.0)) return p.L_ode * Q;
+    if (b == fpow::bits_of(1.0)) return p.L_ode;
+    const int e = (int)(b >> 52) - 1023;
+    if (e >= 2 && e <= 3 && (b & (0x000fffffffffffffull >> e)) == 0) {  // 4 <= b_Psi < 16, an integer
+      const int m = (int)((b & 0x000fffffffffffffull) >> (52 - e)) + (1 << e) - 1;
+      double r = Q;
+      for (int i = 1; i < m; ++i) r *= Q;
+      return p.L_ode * r;
+    }
+    return p.L_ode * fpow::pow_pos(Q, p.b_Psi - 1.0);
+  }
+  AD_HD void rate(const LawParams<double>& p, const double (&v)[5], double (&k)[5]) const {
+    const double L = lambda(p, v);
+#pragma unroll
+    for (int a = 0; a < 5; ++a) k[a] = fma(-L, v[a], ed[a]);
+  }
+  AD_HD void stress(const LawParams<double>& p, double hyd, const double (&v)[5], double (&s)[6]) const {
+    const double m2 = p.mu + p.mu;
+    s[0] = fma(m2, v[0], hyd);
+    s[1] = fma(m2, v[1], hyd);
+    s[2] = fma(-m2, v[0] + v[1], hyd);
+    s[3] = p.mu * v[2];
+    s[4] = p.mu * v[3];
+    s[5] = p.mu * v[4];
+  }
+
+  AD_HD void init(const LawParams<double>& p, const double (&e0_)[6], const double (&e1_)[6], const double (&zn)[6],
+                  const Step& hs, const void* = nullptr) {
+    const double kappa = p.lam + p.mu * (2.0 / 3.0), inv_h = hs.inv_h;
+    const double tr0 = e0_[0] + e0_[1] + e0_[2];
+    double d[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) d[i] = e1_[i] - e0_[i];
+    const double dtr = d[0] + d[1] + d[2];
+    hyd0 = kappa * tr0;
+    dhyd = kappa * dtr;
+    const double yn[5] = {zn[0], zn[1], zn[3], zn[4], zn[5]};
+#pragma unroll
+    for (int a = 0; a < 5; ++a) {
+      e0[a] = a < 2 ? fma(tr0, -1.0 / 3.0, e0_[a]) : e0_[a + 1];
+      de[a] = a < 2 ? fma(dtr, -1.0 / 3.0, d[a]) : d[a + 1];
+      ed[a] = de[a] * inv_h;
+      x[a] = e0[a] - yn[a];
+    }
+    rate(p, x, k1);
+    stress(p, hyd0, x, sig_old);
+    t = 0.0;
+    dt = hs.h;
+    n_acc = n_rej = 0;
+    flags = 0;
+    last_rejected = false;
+    done = false;
+  }
+
+  AD_HD void attempt(const LawParams<double>& p, const Step& hs, const Ode23Ctl& ctl) {
+    const double h = hs.h;
+    if (n_acc + n_rej >= ctl.max_steps) {
+      flags |= ST_CAP;
+      done = true;
+      return;
+    }
+    const bool clip = t + dt >= h;  // the substep that ends the interval ends at h exactly
+    if (clip) dt = h - t;
+    const double tn1 = clip ? h : t + dt;
+    const double th1 = clip ? 1.0 : tn1 * hs.inv_h;
+    double xn[5], e[5], k[5], v[5];
+    if constexpr (PAIR == ERK_BS23) {
+      constexpr double b1 = 2.0 / 9.0, b2 = 1.0 / 3.0, b3 = 4.0 / 9.0;
+      constexpr double e1 = 2.0 / 9.0 - 7.0 / 24.0, e2 = 1.0 / 3.0 - 1.0 / 4.0, e3 = 4.0 / 9.0 - 1.0 / 3.0,
+                       e4 = -1.0 / 8.0;
+      const double c2 = 0.5 * dt, c3 = 0.75 * dt;
+#pragma unroll
+      for (int a = 0; a < 5; ++a) {
+        v[a] = fma(c2, k1[a], x[a]);
+        xn[a] = b1 * k1[a];
+        e[a] = e1 * k1[a];
+      }
+      rate(p, v, k);
+#pragma unroll
+      for (int a = 0; a < 5; ++a) {
+        v[a] = fma(c3, k[a], x[a]);
+        xn[a] = fma(b2, k[a], xn[a]);
+        e[a] = fma(e2, k[a], e[a]);
+      }
+      rate(p, v, k);
+#pragma unroll
+      for (int a = 0; a < 5; ++a) {
+        xn[a] = fma(dt, fma(b3, k[a], xn[a]), x[a]);
+        e[a] = fma(e3, k[a], e[a]);
+      }
+      rate(p, xn, k);  // k1 of the next substep
+#pragma unroll
+      for (int a = 0; a < 5; ++a) e[a] = fma(e4, k[a], e[a]);
+    } else {
+      // Heun (order 2) continued, explicit Euler embedded: difference dt/2 (k2 - k1)
+#pragma unroll
+      for (int a = 0; a < 5; ++a) v[a] = fma(dt, k1[a], x[a]);
+      rate(p, v, k);
+#pragma unroll
+      for (int a = 0; a < 5; ++a) {
+        xn[a] = fma(0.5 * dt, k1[a] + k[a], x[a]);
+        e[a] = 0.5 * (k[a] - k1[a]);
+      }
+      rate(p, xn, k);
+    }
+    double s[6];
+    stress(p, fma(th1, dhyd, hyd0), xn, s);
+    // stress difference of the pair (the hydrostatic parts are the same)
+    const double md = p.mu * dt, m2d = md + md;
+    const double d[6] = {m2d * e[0], m2d * e[1], -m2d * (e[0] + e[1]), md * e[2], md * e[3], md * e[4]};
+    double sum = 0.0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) sum += scaled_sq(d[i], fma(ctl.rtol, absmax_bits(sig_old[i], s[i]), ctl.atol));
+    // err^2, err the RMS; a trial step that overflows is rejected like one with a large error
+    const double err2 = finite64(sum) ? sum * (1.0 / 6.0) : 1e300;
+    // 0.9 err^(-1/3) (ode23), 0.9 err^(-1/2) (ode12)
+    const double f = err2 == 0.0 ? 1e300 : 0.9 * fpow::pow_pos(err2, PAIR == ERK_BS23 ? -1.0 / 6.0 : -1.0 / 4.0);
+    const double grow = fmin(last_rejected ? 1.0 : 5.0, fmax(0.2, f));
+    if (err2 <= 1.0) {
+      t = tn1;
+#pragma unroll
+      for (int a = 0; a < 5; ++a) {
+        x[a] = xn[a];
+        k1[a] = k[a];
+      }
+#pragma unroll
+      for (int i = 0; i < 6; ++i) sig_old[i] = s[i];
+      ++n_acc;
+      last_rejected = false;
+      if (clip) done = true;
+    } else {
+      ++n_rej;
+      last_rejected = true;
+    }
+    dt *= grow;
+  }
+
+  AD_HD unsigned finish(double h, double (&sig)[6], double (&z)[6], double*) const {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) sig[i] = sig_old[i];
+    const double th = t >= h ? 1.0 : t / h;
+    double y[5];
+#pragma unroll
+    for (int a = 0; a < 5; ++a) y[a] = fma(th, de[a], e0[a]) - x[a];
+    z[0] = y[0];
+    z[1] = y[1];
+    z[2] = -(y[0] + y[1]);
+    z[3] = y[2];
+    z[4] = y[3];
+    z[5] = y[4];
+    unsigned st = flags;
+    if (t >= h && !(flags & ST_CAP)) st |= ST_CONVERGED;
+    if (!finite64(sig[0]) || !finite64(z[0])) st |= ST_NONFINITE;
+    st |= (unsigned)(n_acc < 0xffff ? n_acc : 0xffff);
+    st |= (unsigned)(n_rej < 0x7ff ? n_rej : 0x7ff) << ST_ODE_REJ_SHIFT;
+    return st;
+  }
+};
+
+}  // namespace gsm
