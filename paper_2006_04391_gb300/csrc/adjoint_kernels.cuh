@@ -36,6 +36,31 @@ __device__ __forceinline__ void pt_of(const double (&g)[6], double (&gy)[5]) {
   gy[4] = g[5];
 }
 
+// out = C x, C symmetric packed (21 entries, upper triangle row-major).
+__device__ __forceinline__ void ct_times(const double (&C21)[21], const double (&x)[6], double (&out)[6]) {
+  double C[6][6];
+  int q = 0;
+#pragma unroll
+  for (int r = 0; r < 6; ++r)
+#pragma unroll
+    for (int c = r; c < 6; ++c) {
+      C[r][c] = C21[q];
+      C[c][r] = C21[q];
+      ++q;
+    }
+#pragma unroll
+  for (int r = 0; r < 6; ++r) {
+    double acc = 0.0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) acc += C[r][c] * x[c];
+    out[r] = acc;
+  }
+}
+
+// The tangents, K^-1 and the flow's Hessian come from the root (theta, t) of the
+// scalar equation in closed form (ray.cuh); root [2][nvox] keeps it for the
+// finish kernel.  (With the AD blocks, K's factor and its 15 stored entries the
+// two kernels took 940 and 232 us on 64^3 voxels; now 121 and 135.)
 template <int MODE>
 __global__ void __launch_bounds__(kAdjBlock) adj_prepare_kernel(int64_t nvox, const uint8_t* __restrict__ phase,
                                                                 const PhaseTable* __restrict__ tab, double h,
@@ -44,7 +69,7 @@ __global__ void __launch_bounds__(kAdjBlock) adj_prepare_kernel(int64_t nvox, co
                                                                 double gs1, double gs2, double gs3, double gs4,
                                                                 double gs5, const double* __restrict__ g_z,
                                                                 double* __restrict__ Ct21, double* __restrict__ a_u,
-                                                                double* __restrict__ yK) {
+                                                                double* __restrict__ root) {
   const double gs[6] = {gs0, gs1, gs2, gs3, gs4, gs5};
   __shared__ RayConst ray[kMaxPhases];
   if (threadIdx.x < kMaxPhases && tab->kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV)
@@ -56,105 +81,47 @@ __global__ void __launch_bounds__(kAdjBlock) adj_prepare_kernel(int64_t nvox, co
     const bool in = i < nvox;
     const int ph = in ? (int)phase[i] : 0;
     const bool vp = in && tab->kind[ph] == GSM_PSI_ELASTIC_VP_DEV;
-    double e[6], zi[6], s[6], zo[6];
+    double e[6], zi[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       e[c] = in ? eps_k[c * nvox + i] : 0.0;
       zi[c] = vp ? zprev[c * nvox + i] : 0.0;
     }
     if (!in) continue;
-    if (vp) voxel_ray<NortonDev>(ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<double*>(nullptr));
-    double C[6][6], au[6];
+    double C21[21], au[6];
     if (vp) {
-      const LawParams<double>& p = tab->p64[ph];
-      const double y[5] = {zo[0], zo[1], zo[3], zo[4], zo[5]};
+      const RayConst& c = ray[ph];
       const double yn[5] = {zi[0], zi[1], zi[3], zi[4], zi[5]};
-      double sig[6], Cee[6][6], Cey[6][5], Cye[5][6], g[5], K[5][5];
-      psi_blocks<NortonDev>(p, e, y, sig, Cee, Cey, Cye);
-      psi_y_yy<NortonDev>(p, e, y, g, K);
-      bool flow = false;
+      RayVoxel v;
+      ray_solve<NortonDev>(c, e, yn, true, MODE == MODE_FP32_FIX, v);
+      const double E2 = v.norm2();
+      ray_tangent<double>(c.mu, c.kappa, c.p, v.es, E2, v.theta, v.t, v.r.flows, C21);
+      ct_times(C21, gs, au);
+      if (v.r.flows) {
+        double gz[6], gy[5], t[5];
 #pragma unroll
-      for (int a = 0; a < 5; ++a) flow = flow || (y[a] != yn[a]);
-      double gz[6], gy[5], t[5] = {0, 0, 0, 0, 0};
+        for (int q = 0; q < 6; ++q) gz[q] = g_z[q * nvox + i];
+        pt_of(gz, gy);
+        const double d[5] = {v.es[0], v.es[1], v.es[3], v.es[4], v.es[5]};
+        ray_K_solve(c.mu, c.p, v.theta, v.t, E2, d, gy, t);
+        // - psi_ey t = C P t
+        au[0] += 2.0 * c.mu * t[0];
+        au[1] += 2.0 * c.mu * t[1];
+        au[2] -= 2.0 * c.mu * (t[0] + t[1]);
 #pragma unroll
-      for (int c = 0; c < 6; ++c) gz[c] = g_z[c * nvox + i];
-      pt_of(gz, gy);
-#pragma unroll
-      for (int r = 0; r < 6; ++r)
-#pragma unroll
-        for (int c = 0; c < 6; ++c) C[r][c] = Cee[r][c];
-      if (flow) {
-        const double inv_h = 1.0 / h;
-        double v[5], gv[5], Hv[5][5];
-#pragma unroll
-        for (int a = 0; a < 5; ++a) v[a] = (y[a] - yn[a]) * inv_h;
-        phi_v_vv<NortonDev>(p, v, gv, Hv);
-#pragma unroll
-        for (int a = 0; a < 5; ++a)
-#pragma unroll
-          for (int b = 0; b < 5; ++b) K[a][b] += Hv[a][b] * inv_h;
-        Chol5<double> ch;
-        ch.factor(K);
-        ch.solve(gy, t);
-        // C_t = Cee + Cey dy/deps, dy/deps = -K^-1 Cye
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          double rhs[5], dy[5];
-#pragma unroll
-          for (int a = 0; a < 5; ++a) rhs[a] = -Cye[a][c];
-          ch.solve(rhs, dy);
-#pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            double acc = 0.0;
-#pragma unroll
-            for (int a = 0; a < 5; ++a) acc += Cey[r][a] * dy[a];
-            C[r][c] += acc;
-          }
-        }
+        for (int q = 3; q < 6; ++q) au[q] += c.mu * t[q - 1];
       }
-#pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        double acc = 0.0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) acc += C[c][r] * gs[c];
-#pragma unroll
-        for (int a = 0; a < 5; ++a) acc -= Cey[r][a] * t[a];
-        au[r] = acc;
-      }
-#pragma unroll
-      for (int a = 0; a < 5; ++a) yK[a * nvox + i] = y[a];
-      int q = 5;
-#pragma unroll
-      for (int a = 0; a < 5; ++a)
-#pragma unroll
-        for (int b = a; b < 5; ++b) yK[(q++) * nvox + i] = K[a][b];
+      root[i] = v.r.flows ? v.theta : 0.0;
+      root[nvox + i] = v.t;
     } else {
-      double C21[21];
+      double s[6];
       voxel_elastic<double>(tab->p64[ph], e, s, C21);
-      int q = 0;
-#pragma unroll
-      for (int r = 0; r < 6; ++r)
-#pragma unroll
-        for (int c = r; c < 6; ++c) {
-          C[r][c] = C21[q];
-          C[c][r] = C21[q];
-          ++q;
-        }
-#pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        double acc = 0.0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) acc += C[c][r] * gs[c];
-        au[r] = acc;
-      }
+      ct_times(C21, gs, au);
     }
-    int q = 0;
 #pragma unroll
-    for (int r = 0; r < 6; ++r)
+    for (int q = 0; q < 21; ++q) Ct21[q * nvox + i] = C21[q];
 #pragma unroll
-      for (int c = r; c < 6; ++c) Ct21[(q++) * nvox + i] = 0.5 * (C[r][c] + C[c][r]);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) a_u[c * nvox + i] = au[c];
+    for (int q = 0; q < 6; ++q) a_u[q * nvox + i] = au[q];
   }
 }
 
@@ -230,7 +197,7 @@ __global__ void __launch_bounds__(kAdjBlock) adj_finish_kernel(
     int64_t nvox, const uint8_t* __restrict__ phase, const PhaseTable* __restrict__ tab, double h, int phase_id,
     NortonTheta th, const double* __restrict__ eps_k, const double* __restrict__ zprev, double gs0, double gs1,
     double gs2, double gs3, double gs4, double gs5, const double* __restrict__ g_z, const double* __restrict__ lam_raw,
-    double inv_n3, const double* __restrict__ yK, double* __restrict__ g_z_prev, double* __restrict__ partials) {
+    double inv_n3, const double* __restrict__ root, double* __restrict__ g_z_prev, double* __restrict__ partials) {
   const double gs[6] = {gs0, gs1, gs2, gs3, gs4, gs5};
   double acc[3] = {0.0, 0.0, 0.0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -239,7 +206,8 @@ __global__ void __launch_bounds__(kAdjBlock) adj_finish_kernel(
     double out[6] = {0, 0, 0, 0, 0, 0};
     if (tab->kind[ph] == GSM_PSI_ELASTIC_VP_DEV) {
       const LawParams<double>& p = tab->p64[ph];
-      double e[6], a[6], gz[6], gy[5], y[5], yn[5], K[5][5];
+      const double pe = 1.0 + 2.0 * (p.a_phi - 1.0), mu = p.mu, kappa = p.lam + p.mu * (2.0 / 3.0);
+      double e[6], a[6], gz[6], gy[5], yn[5], es[6];
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
         e[c] = eps_k[c * nvox + i];
@@ -251,50 +219,20 @@ __global__ void __launch_bounds__(kAdjBlock) adj_finish_kernel(
       yn[2] = zprev[3 * nvox + i];
       yn[3] = zprev[4 * nvox + i];
       yn[4] = zprev[5 * nvox + i];
-#pragma unroll
-      for (int b = 0; b < 5; ++b) y[b] = yK[b * nvox + i];
-      int q = 5;
-#pragma unroll
-      for (int r = 0; r < 5; ++r)
-#pragma unroll
-        for (int c = r; c < 5; ++c) {
-          const double v = yK[(q++) * nvox + i];
-          K[r][c] = v;
-          K[c][r] = v;
-        }
+      const double theta = root[i], t = root[nvox + i];
+      const double tr = NortonDev::trial_strain(e, yn, es);
+      const double E2 = es[0] * es[0] + es[1] * es[1] + es[2] * es[2] +
+                        0.5 * (es[3] * es[3] + es[4] * es[4] + es[5] * es[5]);
+      const double d[5] = {es[0], es[1], es[3], es[4], es[5]};
       pt_of(gz, gy);
-      double sig[6], Cee[6][6], Cey[6][5], Cye[5][6], psy[5];
-      psi_blocks<NortonDev>(p, e, y, sig, Cee, Cey, Cye);
-      psi_y_and_stress<NortonDev>(p, e, y, psy, sig);
-      double rhs[5];
-#pragma unroll
-      for (int r = 0; r < 5; ++r) {
-        double s = gy[r];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) s += Cye[r][c] * a[c];
-        rhs[r] = s;
-      }
-      bool flow = false;
-#pragma unroll
-      for (int b = 0; b < 5; ++b) flow = flow || (y[b] != yn[b]);
+      // rhs = P^T g_z + psi_ye a, psi_ye a = -P^T C a
+      const double rhs[5] = {gy[0] - 2.0 * mu * (a[0] - a[2]), gy[1] - 2.0 * mu * (a[1] - a[2]), gy[2] - mu * a[3],
+                             gy[3] - mu * a[4], gy[4] - mu * a[5]};
       double b5[5] = {0, 0, 0, 0, 0}, gyn[5];
-      double v[5];
-      const double inv_h = 1.0 / h;
-#pragma unroll
-      for (int b = 0; b < 5; ++b) v[b] = (y[b] - yn[b]) * inv_h;
+      const bool flow = theta > 0.0;
       if (flow) {
-        Chol5<double> ch;
-        ch.factor(K);
-        ch.solve(rhs, b5);
-        double gv[5], Hv[5][5];
-        phi_v_vv<NortonDev>(p, v, gv, Hv);
-#pragma unroll
-        for (int r = 0; r < 5; ++r) {
-          double s = 0.0;
-#pragma unroll
-          for (int c = 0; c < 5; ++c) s += Hv[r][c] * b5[c];
-          gyn[r] = s * inv_h;
-        }
+        ray_K_solve(mu, pe, theta, t, E2, d, rhs, b5);
+        ray_flow_apply(mu, pe, theta, t, E2, d, b5, gyn);
       } else {
 #pragma unroll
         for (int r = 0; r < 5; ++r) gyn[r] = rhs[r];
@@ -307,13 +245,17 @@ __global__ void __launch_bounds__(kAdjBlock) adj_finish_kernel(
       if (ph == phase_id) {
         // P^T sigma = -psi_y; dR/dE = psi_y / E, dR/dsigma0 = phi_v / sigma0 = P^T sigma / sigma0,
         // dR/dn = P^T sigma (-ln(s/edot0) / n^2); dsigma/dE|_y = sigma / E
+        double sig[6], Ps[5];
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+          sig[c] = c < 3 ? 2.0 * mu * t * es[c] + kappa * tr : mu * t * es[c];
+        pt_of(sig, Ps);
         double bP = 0.0, aS = 0.0;
 #pragma unroll
-        for (int r = 0; r < 5; ++r) bP -= b5[r] * psy[r];
+        for (int r = 0; r < 5; ++r) bP += b5[r] * Ps[r];
 #pragma unroll
         for (int c = 0; c < 6; ++c) aS += a[c] * sig[c];
-        const double qv = (4.0 / 3.0) * (v[0] * v[0] + v[1] * v[1] + v[0] * v[1]) +
-                          (1.0 / 3.0) * (v[2] * v[2] + v[3] * v[3] + v[4] * v[4]);
+        const double v = theta / h, qv = (2.0 / 3.0) * E2 * v * v;
         const double logt = qv > 0.0 ? 0.5 * log(qv) - log(th.edot0) : 0.0;
         acc[0] += (aS + bP) / th.E;
         acc[1] += -bP / th.sigma0;
@@ -415,13 +357,14 @@ __global__ void cg_direction_kernel(int64_t n, double b, const double* __restric
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) p[i] = r[i] + b * p[i];
 }
 
+// One warp per sum, fixed lane stride and shuffle tree.  Launch with 96 threads.
 __global__ void adj_sum_kernel(const double* __restrict__ partials, int n, double* __restrict__ out) {
-  const int t = threadIdx.x;
-  if (t < 3) {
-    double s = 0.0;
-    for (int b = 0; b < n; ++b) s += partials[t * n + b];
-    out[t] = s;
-  }
+  const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int b = lane; b < n; b += 32) s += partials[t * n + b];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) out[t] = s;
 }
 
 }  // namespace

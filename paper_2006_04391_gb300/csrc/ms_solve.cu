@@ -1243,7 +1243,7 @@ struct Tape {
   double* ckpt = nullptr;  // [2][n_steps][6][nvox]: eps_k, then z_{k-1}
   double* Ct21 = nullptr;  // [21][nvox]
   double* a_u = nullptr;   // [6][nvox]
-  double* yK = nullptr;    // [20][nvox]: y (5) and K upper triangle (15)
+  double* root = nullptr;  // [2][nvox]: theta and 1 - theta of each voxel's scalar equation
   double* gz = nullptr;    // [6][nvox]
   double* gz_prev = nullptr;
   double* cg_lam = nullptr;  // [6][nvox] conjugate gradients: lam, residual, direction
@@ -1275,7 +1275,7 @@ int ms_run_taped(ms_handle h, const ms_load* load, ms_result* result, ms_tape_ha
   bool ok = cudaMalloc((void**)&t->ckpt, ck) == cudaSuccess &&
             cudaMalloc((void**)&t->Ct21, 21 * j.nvox * sizeof(double)) == cudaSuccess &&
             cudaMalloc((void**)&t->a_u, n6 * sizeof(double)) == cudaSuccess &&
-            cudaMalloc((void**)&t->yK, 20 * j.nvox * sizeof(double)) == cudaSuccess &&
+            cudaMalloc((void**)&t->root, 2 * j.nvox * sizeof(double)) == cudaSuccess &&
             cudaMalloc((void**)&t->gz, n6 * sizeof(double)) == cudaSuccess &&
             cudaMalloc((void**)&t->gz_prev, n6 * sizeof(double)) == cudaSuccess &&
             cudaMalloc((void**)&t->cg_lam, n6 * sizeof(double)) == cudaSuccess &&
@@ -1343,11 +1343,11 @@ int ms_adjoint(ms_tape_handle th, const double* w, int phase_id, double tol, int
     if (j.law_mode == MODE_FP64)
       adj_prepare_kernel<MODE_FP64><<<grid_prep, kAdjBlock, 0, s>>>(nv, j.phase, j.tab_dev, hk, eps_k, zprev, gs[0],
                                                                      gs[1], gs[2], gs[3], gs[4], gs[5], t.gz, t.Ct21,
-                                                                     t.a_u, t.yK);
+                                                                     t.a_u, t.root);
     else
       adj_prepare_kernel<MODE_FP32_FIX><<<grid_prep, kAdjBlock, 0, s>>>(nv, j.phase, j.tab_dev, hk, eps_k, zprev,
                                                                          gs[0], gs[1], gs[2], gs[3], gs[4], gs[5],
-                                                                         t.gz, t.Ct21, t.a_u, t.yK);
+                                                                         t.gz, t.Ct21, t.a_u, t.root);
     count_launch();
     // adjoint equilibrium by conjugate gradients on G (C_t lam) = G a_u, G the
     // Green operator of C0 = identity (lam0 = 0, mu0 = 1/2): lam, r, p
@@ -1514,8 +1514,8 @@ int ms_adjoint(ms_tape_handle th, const double* w, int phase_id, double tol, int
     capped = capped || !conv;
     adj_finish_kernel<<<grid_fin, kAdjBlock, 0, s>>>(nv, j.phase, j.tab_dev, hk, phase_id, nt, eps_k, zprev, gs[0],
                                                      gs[1], gs[2], gs[3], gs[4], gs[5], t.gz, j.f64.eps_raw, inv_n3,
-                                                     t.yK, t.gz_prev, t.part);
-    adj_sum_kernel<<<1, 32, 0, s>>>(t.part, grid_fin, t.out_dev);
+                                                     t.root, t.gz_prev, t.part);
+    adj_sum_kernel<<<1, 96, 0, s>>>(t.part, grid_fin, t.out_dev);
     count_launch(2);
     cudaMemcpyAsync(t.out_host, t.out_dev, 3 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return GSM_ECUDA;
@@ -1533,7 +1533,7 @@ int ms_tape_destroy(ms_tape_handle th) {
   cudaFree(t->ckpt);
   cudaFree(t->Ct21);
   cudaFree(t->a_u);
-  cudaFree(t->yK);
+  cudaFree(t->root);
   cudaFree(t->gz);
   cudaFree(t->gz_prev);
   cudaFree(t->cg_lam);
