@@ -30,11 +30,14 @@
  *     crosses the ABI.  gsm_strerror() gives a static message.
  *
  * Per-voxel status word (int32, optional output of gsm_update):
- *   bits 0-7 line-search iterations, bits 8-15 Newton iterations (including
- *   FP64 corrections), bit 16 converged, bit 17 non-finite input or result,
+ *   bits 0-7 line-search iterations (evaluations of the segment function in the
+ *   working precision), bits 8-15 Newton iterations (including FP64
+ *   corrections), bit 16 converged, bit 17 non-finite input or result,
  *   bit 18 iteration cap reached, bit 19 Newton matrix not positive definite,
  *   bits 20-23 FP64 corrections (GSM_FP32_FP64FIX), bits 24-30 scalar
- *   iterations of the segment model that starts the line search.
+ *   iterations of the segment model that starts the line search.  The Norton
+ *   law's step has its root on the predictor segment: it takes scalar iterations
+ *   (FP32) and one evaluation there, no Newton iteration of the full system.
  */
 #ifndef GSM_GB300_H
 #define GSM_GB300_H
@@ -64,8 +67,9 @@ extern "C" {
 #define GSM_PHI_MS_FORCE 2       /* Eq. michel_suquet_psi (a FORCE potential Psi(A)):
                                     sigma_d edot0/(n+1) ((|dev A_z|_eq + A_alpha)^+/sigma_d)^(n+1) */
 
-#define GSM_FP64 0               /* every step in FP64                                 */
-#define GSM_FP32_FP64FIX 1       /* FP32 Newton, then FP64 correction (FP64 in/out)    */
+#define GSM_FP64 0               /* solved and evaluated in FP64 (FP32 starting values) */
+#define GSM_FP32_FP64FIX 1       /* FP32 solve, then one correction whose residual has
+                                    double-float (2^-45) accuracy (FP64 in/out)        */
 #define GSM_FP32 2               /* FP32 in, out and arithmetic                        */
 
 typedef struct gsm_material* gsm_handle;
@@ -120,15 +124,17 @@ int gsm_update(gsm_handle h, int64_t n_vox, const void* eps, const void* z_n, in
                void* sigma, void* z, void* tangent, int32_t* status, void* stream);
 
 /*
- * gsm_update_host -- gsm_update for arrays that live in page-locked host memory,
- * streamed through the device in chunks of `chunk` voxels (0: 2^20): the
+ * gsm_update_host -- gsm_update for arrays that live in page-locked host memory.
+ * chunk = 0: the kernel reads and writes them directly over the host link (as
+ * gsm_update does), or, where the device cannot address them, in chunks of 2^17.
+ * chunk > 0: streamed through the device in chunks of `chunk` voxels: the
  * host->device copies of chunk i+1 and the device->host copies of chunk i-1
  * (two internal streams, the copy engines of both directions of the host link)
  * overlap the update of chunk i (on `stream`).  Same arguments, layouts and
  * results as gsm_update (bit-identical to it on device copies of the arrays);
  * every non-NULL array must be page-locked host memory (cudaHostAlloc /
- * cudaHostRegister), else GSM_EINVAL.  Device staging buffers for three
- * chunks come from the stream-ordered allocator of the current device and go
+ * cudaHostRegister), else GSM_EINVAL.  When streaming, device staging buffers
+ * for three chunks come from the stream-ordered allocator of the current device and go
  * back to it on `stream`.  Asynchronous on `stream`: the results are in host
  * memory once `stream` has passed this call.  Errors: GSM_EINVAL, GSM_ENOMEM,
  * GSM_ENOTSUP, GSM_ECUDA.
@@ -216,10 +222,10 @@ int gsm_peak_probe(int precision, int64_t iters, int blocks_per_sm, double* fmas
  * (fixed C^ref, Sec. 3).  Load step k: eps <- eps + (E_k - E_{k-1}), then
  * iterate
  *     sigma = law(eps, z_n, h_k)               (material kernel)
- *     sigma^ = FFT(sigma)                      (cuFFT R2C)
+ *     sigma^ = FFT(sigma)                      (real to complex)
  *     e = sqrt(sum_xi |xi.sigma^/N^3|^2) / |<sigma>|_F   (FP64 reduction)
  *     eps^(xi) -= Gamma0(xi) : sigma^(xi), eps^(0) = N^3 E_k   (fused kernel)
- *     eps = IFFT(eps^)                         (cuFFT C2R)
+ *     eps = IFFT(eps^)                         (complex to real)
  * until e < tol; then z_n <- z and Sigma_k = <sigma> (FP64).  xi = 2 pi k with
  * k the signed integer frequency; on even grids a mode with the Nyquist index
  * together with any other nonzero index has Gamma0 := 0 and is left out of e.
@@ -368,10 +374,10 @@ int ms_tape_destroy(ms_tape_handle tape);
 /* ===================================================== serving (batched jobs)
  *
  * A server keeps many basic-scheme jobs resident on one GPU and advances the
- * active jobs by one iteration per serve_tick: one material launch, one
- * Green-operator launch and one reduction launch cover every job of the tick
- * (per-job cuFFT calls in between), then one device-to-host copy of their
- * errors.  Jobs that arrive while others run are admitted first come first
+ * active jobs by one iteration per serve_tick: one material launch covers every
+ * job of the tick, one launch per transform pass every job of one grid size
+ * (grid sizes without the library's own transforms: cuFFT per job), and the
+ * errors are written to host memory.  Jobs that arrive while others run are admitted first come first
  * served at the next tick when a slot (max_active) and the HBM budget allow;
  * finished jobs release their memory at once.  Which active jobs a tick takes
  * is fair share: each job carries the GPU work it has received (N^3 per FP32
