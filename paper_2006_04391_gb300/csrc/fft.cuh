@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
     __syncthreads();
     if (last) {
       __threadfence();
-      finalize_sums(v.mat_part, v.n_vch, v.gam_part, tiles, v.inv_n3, v.mu0 * 1e-6, v.red);
+      finalize_sums(v.mat_part, v.n_vch, v.gam_part, tiles, v.inv_n3, v.mu0 * 1e-6, v.red, v.mean);
       if (threadIdx.x == 0) *v.arrived = 0u;
     }
   }

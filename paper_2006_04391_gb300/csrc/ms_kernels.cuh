@@ -59,15 +59,17 @@ struct JobView {
   RayConst ray[kMaxPhases];  // the scalar equation of each Norton phase at this step's h
   int kind[kMaxPhases];      // GSM_PSI_* of each phase
   const uint8_t* phase;
-  const void* eps_raw;   // [6][nvox] N^3 * strain (C2R output)
+  const void* eps_raw;   // [6][nvox] N^3 * strain (inverse transform's output); FP32 fields: without its mean
   const void* zn;        // [6][nvox]
-  void* sig;             // [6][nvox]
+  void* sig;             // [6][nvox] stress; FP32 fields: less the mean stress of the evaluation before
   void* eps_out;         // [6][nvox] where the inverse transform writes the next strain
   void* z;               // [6][nvox]
   void* sig_hat;         // [6][nmodes]
   void* eps_hat;         // [6][nmodes]
   double* mat_part;      // [6][n_vch]
   double* gam_part;      // [n_mch]
+  double* mean;          // [6] the mean stress of the job's last evaluation (device)
+  double E[6];           // mean strain
   Reduced* red;          // where the job's error and mean stress go (page-locked host memory)
   unsigned* arrived;     // blocks of the fused Green pass that are done (0 between launches), or NULL
   const PhaseTable* tab;
@@ -164,9 +166,16 @@ __device__ __forceinline__ void block_sum6_at(const double (&v)[6], double* out,
 }
 
 // The laws of a job's phases as the material kernels read them (shared memory).
+//
+// FP32 fields hold what varies: the strain without its mean E (added here as a
+// pair of FP32 numbers) and the stress less a uniform one (the mean of the
+// evaluation before; the Green operator does not see the zero mode).  Their
+// rounding, and that of the transforms, is then relative to the fluctuations
+// and not to the means.
 struct LawTable {
   RayConst ray[kMaxPhases];
   int kind[kMaxPhases];
+  float E_hi[6], E_lo[6], sub[6];
 };
 
 // Material evaluation of voxel i.  The field precision T is also that of the
@@ -186,7 +195,10 @@ __device__ __forceinline__ void material_voxel(int64_t i, int64_t nvox, const ui
 #pragma unroll
   for (int c = 0; c < 6; ++c) zi[c] = __ldg(zn + c * nvox + i);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) e[c] *= inv_n3;
+  for (int c = 0; c < 6; ++c) {
+    if constexpr (sizeof(T) == 4) e[c] = fmaf(e[c], inv_n3, law.E_lo[c]) + law.E_hi[c];
+    else e[c] *= inv_n3;
+  }
   if (law.kind[ph] == GSM_PSI_ELASTIC_VP_DEV) {
     voxel_ray<NortonDev>(law.ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<T*>(nullptr));
   } else {
@@ -195,7 +207,8 @@ __device__ __forceinline__ void material_voxel(int64_t i, int64_t nvox, const ui
   }
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
-    sig[c * nvox + i] = s[c];
+    if constexpr (sizeof(T) == 4) sig[c * nvox + i] = s[c] - law.sub[c];
+    else sig[c * nvox + i] = s[c];
     z[c * nvox + i] = zo[c];
     acc[c] += s[c];
   }
@@ -403,6 +416,12 @@ __global__ void __launch_bounds__(kMatBlock) ms_material_batch_kernel(const JobV
       int* dst = reinterpret_cast<int*>(law.ray);
       for (int k = threadIdx.x; k < v.n_phases * (int)(sizeof(RayConst) / 4); k += blockDim.x) dst[k] = src[k];
       if (threadIdx.x < kMaxPhases) law.kind[threadIdx.x] = v.kind[threadIdx.x];
+      if (sizeof(T) == 4 && threadIdx.x < 6) {
+        const double E = v.E[threadIdx.x];
+        law.E_hi[threadIdx.x] = (float)E;
+        law.E_lo[threadIdx.x] = (float)(E - (double)(float)E);
+        law.sub[threadIdx.x] = (float)v.mean[threadIdx.x];
+      }
       held = job;
       __syncthreads();
     }
@@ -464,7 +483,8 @@ __global__ void __launch_bounds__(kGamBlock) ms_gamma_batch_kernel(const JobView
 // problems in a batch).  The 256^3 sums took 58 us with one warp a sum.
 constexpr int kFinBlock = 512;
 __device__ void finalize_sums(const double* __restrict__ mat_part, int n_mat, const double* __restrict__ gam_part,
-                              int n_gam, double inv_n3, double floor_, Reduced* __restrict__ out) {
+                              int n_gam, double inv_n3, double floor_, Reduced* __restrict__ out,
+                              double* __restrict__ mean = nullptr) {
   __shared__ double sum[7];
   double a[7] = {0, 0, 0, 0, 0, 0, 0};
 #pragma unroll 4
@@ -482,6 +502,8 @@ __device__ void finalize_sums(const double* __restrict__ mat_part, int n_mat, co
     const double fro = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2] + 2.0 * (m[3] * m[3] + m[4] * m[4] + m[5] * m[5]));
     out->e = num / fmax(fro, floor_);
     for (int c = 0; c < 6; ++c) out->mean[c] = m[c];
+    if (mean)
+      for (int c = 0; c < 6; ++c) mean[c] = m[c];
     out->res = sum[6];
   }
 }
@@ -495,7 +517,7 @@ __global__ void ms_finalize_kernel(const double* __restrict__ mat_part, int n_ma
 // One block per job.
 __global__ void ms_finalize_batch_kernel(const JobView* __restrict__ views) {
   const JobView& v = views[blockIdx.x];
-  finalize_sums(v.mat_part, v.n_vch, v.gam_part, v.n_mch, v.inv_n3, v.mu0 * 1e-6, v.red);
+  finalize_sums(v.mat_part, v.n_vch, v.gam_part, v.n_mch, v.inv_n3, v.mu0 * 1e-6, v.red, v.mean);
 }
 
 // Mean mode of the strain spectrum and of the inverse-transform input:
@@ -605,6 +627,16 @@ __global__ void ms_add_uniform_kernel(int64_t nvox, T* __restrict__ eps_raw, dou
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += stride)
 #pragma unroll
     for (int c = 0; c < 6; ++c) eps_raw[c * nvox + i] = (T)((double)eps_raw[c * nvox + i] + d[c]);
+}
+
+// dst = src + off, one offset a component, with conversion (the FP32 strain
+// without its mean and back).
+template <class S, class D>
+__global__ void ms_offset_convert_kernel(int64_t nvox, const S* __restrict__ src, D* __restrict__ dst, double6 off) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += stride)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) dst[c * nvox + i] = (D)((double)src[c * nvox + i] + off.v[c]);
 }
 
 // eps_hat = R2C(eps_raw) / N^3 with the mean mode set to N^3 E exactly.

@@ -250,6 +250,7 @@ struct Job {
   double* mat_part = nullptr;
   double* gam_part = nullptr;
   unsigned* arrived = nullptr;       // counter of the fused Green pass
+  double* mean_dev = nullptr;        // [6] mean stress of the last evaluation
   size_t bytes = 0;
   bool allocated = false;
   // load
@@ -351,7 +352,9 @@ void job_free(Job& j, cudaStream_t s) {
   if (j.mat_part) cudaFreeAsync(j.mat_part, s);
   if (j.gam_part) cudaFreeAsync(j.gam_part, s);
   if (j.arrived) cudaFreeAsync(j.arrived, s);
+  if (j.mean_dev) cudaFreeAsync(j.mean_dev, s);
   j.arrived = nullptr;
+  j.mean_dev = nullptr;
   if (j.tab_dev) cudaFreeAsync(j.tab_dev, s);
   if (j.phase_owned) cudaFreeAsync(j.phase_owned, s);
   if (j.eps_prev) cudaFreeAsync(j.eps_prev, s);
@@ -373,6 +376,8 @@ int job_alloc(Job& j, cudaStream_t s, const uint8_t* phase_host) {
        cudaMallocAsync((void**)&j.gam_part, (size_t)n_gam_part(j.N) * sizeof(double), s) == cudaSuccess &&
        cudaMallocAsync((void**)&j.arrived, sizeof(unsigned), s) == cudaSuccess &&
        cudaMemsetAsync(j.arrived, 0, sizeof(unsigned), s) == cudaSuccess &&
+       cudaMallocAsync((void**)&j.mean_dev, 6 * sizeof(double), s) == cudaSuccess &&
+       cudaMemsetAsync(j.mean_dev, 0, 6 * sizeof(double), s) == cudaSuccess &&
        cudaMallocAsync((void**)&j.tab_dev, sizeof(PhaseTable), s) == cudaSuccess;
   if (ok && phase_host) {
     ok = cudaMallocAsync((void**)&j.phase_owned, (size_t)j.nvox, s) == cudaSuccess &&
@@ -497,21 +502,38 @@ template <class S, class D> void convert(cudaStream_t s, const S* src, D* dst, i
   count_launch();
 }
 
-// eps_raw += N^3 (E - E_prev); eps_hat = spectrum of eps with mean N^3 E.
+template <class S, class D> void offset_convert(cudaStream_t s, const S* src, D* dst, int64_t nvox, const double (&off)[6]) {
+  double6 o;
+  for (int q = 0; q < 6; ++q) o.v[q] = off[q];
+  ms_offset_convert_kernel<S, D><<<elt_grid(nvox), 256, 0, s>>>(nvox, src, dst, o);
+  count_launch();
+}
+
+// FP64 fields: eps_raw += N^3 (E - E_prev); eps_hat = spectrum of eps with mean
+// N^3 E.  FP32 fields hold the strain without its mean: their spectrum's mean
+// mode is 0.
 template <class T> int spectrum_start(Engine& g, Job& j, const double* E, const double* E_prev) {
   Fields<T>& f = fields<T>(j);
   Plans* p = nullptr;
   int rc = g.get_plans(j.N, sizeof(T) == 4, &p);
   if (rc != GSM_OK) return rc;
   const double n3 = (double)j.nvox;
-  double d[6];
-  for (int q = 0; q < 6; ++q) d[q] = n3 * (E[q] - E_prev[q]);
-  ms_add_uniform_kernel<T><<<elt_grid(j.nvox), 256, 0, g.stream>>>(j.nvox, f.eps_raw, d[0], d[1], d[2], d[3], d[4],
-                                                                     d[5]);
+  double m[6] = {0, 0, 0, 0, 0, 0};
+  if (sizeof(T) == 8) {
+    double d[6];
+    for (int q = 0; q < 6; ++q) {
+      d[q] = n3 * (E[q] - E_prev[q]);
+      m[q] = E[q];
+    }
+    ms_add_uniform_kernel<T><<<elt_grid(j.nvox), 256, 0, g.stream>>>(j.nvox, f.eps_raw, d[0], d[1], d[2], d[3], d[4],
+                                                                       d[5]);
+    count_launch();
+  }
   if (!exec_r2c(*p, f.eps_raw, f.sig_hat, g.stream)) return GSM_ECUDA;
-  ms_spectrum_init_kernel<T><<<elt_grid(j.nmodes), 256, 0, g.stream>>>(j.nmodes, f.sig_hat, f.eps_hat, (p->ops ? 0.5 : 1.0) / n3, n3,
-                                                                         E[0], E[1], E[2], E[3], E[4], E[5]);
-  count_launch(2);
+  ms_spectrum_init_kernel<T><<<elt_grid(j.nmodes), 256, 0, g.stream>>>(j.nmodes, f.sig_hat, f.eps_hat,
+                                                                         (p->ops ? 0.5 : 1.0) / n3, n3, m[0], m[1], m[2],
+                                                                         m[3], m[4], m[5]);
+  count_launch();
   return cudaGetLastError() == cudaSuccess ? GSM_OK : GSM_ECUDA;
 }
 
@@ -629,7 +651,9 @@ int step_start(Engine& g, Job& j) {
   j.since_best = 0;
   j.fp32_phase = j.precision == MS_PREC_FP32_BULK && cap_of(j) > 1;
   if (j.fp32_phase) {
-    convert<double, float>(g.stream, j.f64.eps_raw, j.f32.eps_raw, 6 * j.nvox, 1.0);
+    double off[6];
+    for (int q = 0; q < 6; ++q) off[q] = -(double)j.nvox * j.E_prev[q];
+    offset_convert<double, float>(g.stream, j.f64.eps_raw, j.f32.eps_raw, j.nvox, off);
     convert<double, float>(g.stream, j.f64.zn, j.f32.zn, 6 * j.nvox, 1.0);
     return spectrum_start<float>(g, j, E, j.E_prev);
   }
@@ -648,14 +672,15 @@ template <class T> int move_mean(Engine& g, Job& j, const double (&dS)[6]) {
     j.E_cur[j.s_idx[a]] += d;
     dm.v[j.s_idx[a]] = n3 * d;
   }
-  for (int q = 0; q < 6; ++q) m.v[q] = n3 * j.E_cur[q];
-  Fields<T>& f = fields<T>(j);
-  Plans* p = nullptr;
-  const int rc = g.get_plans(j.N, sizeof(T) == 4, &p);
-  if (rc != GSM_OK) return rc;
-  if (p->ops) ms_move_mean_kernel<T><<<1, 256, 0, g.stream>>>(f.eps_hat, f.sig_hat, j.N, m, dm);
-  else ms_set_mean_kernel<T><<<1, 32, 0, g.stream>>>(f.eps_hat, f.sig_hat, j.nmodes, m);
-  count_launch();
+  if constexpr (sizeof(T) == 8) {  // (the mean strain is not in the FP32 fields)
+    for (int q = 0; q < 6; ++q) m.v[q] = n3 * j.E_cur[q];
+    Plans* p = nullptr;
+    const int rc = g.get_plans(j.N, false, &p);
+    if (rc != GSM_OK) return rc;
+    if (p->ops) ms_move_mean_kernel<double><<<1, 256, 0, g.stream>>>(j.f64.eps_hat, j.f64.sig_hat, j.N, m, dm);
+    else ms_set_mean_kernel<double><<<1, 32, 0, g.stream>>>(j.f64.eps_hat, j.f64.sig_hat, j.nmodes, m);
+    count_launch();
+  }
   return GSM_OK;
 }
 
@@ -663,7 +688,9 @@ template <class T> int move_mean(Engine& g, Job& j, const double (&dS)[6]) {
 // evaluation becomes the FP64 strain, resynthesised from its spectrum so that
 // its mean is E_k exactly.
 int switch_to_fp64(Engine& g, Job& j) {
-  convert<float, double>(g.stream, j.f32.eps_raw, j.f64.eps_raw, 6 * j.nvox, 1.0);
+  double off[6];
+  for (int q = 0; q < 6; ++q) off[q] = (double)j.nvox * j.E_cur[q];
+  offset_convert<float, double>(g.stream, j.f32.eps_raw, j.f64.eps_raw, j.nvox, off);
   int rc = spectrum_start<double>(g, j, j.E_cur, j.E_cur);
   if (rc != GSM_OK) return rc;
   cudaMemcpyAsync(j.f64.sig_hat, j.f64.eps_hat, 6 * j.nmodes * sizeof(cufftDoubleComplex), cudaMemcpyDeviceToDevice,
@@ -803,6 +830,8 @@ int tick(Engine& g, const std::vector<Job*>& jobs) {
     v.eps_out = v.sig;  // (the stress is not needed once its spectrum is formed)
     v.mat_part = j.mat_part;
     v.gam_part = j.gam_part;
+    v.mean = j.mean_dev;
+    for (int q = 0; q < 6; ++q) v.E[q] = j.E_cur[q];
     v.red = g.red_host + i;
     v.arrived = plan[i]->ops ? j.arrived : nullptr;
     v.tab = j.tab_dev;
@@ -913,7 +942,7 @@ int tick(Engine& g, const std::vector<Job*>& jobs) {
     for (int q = i; p.ops && q < e; ++q) {
       Job& j = *order[q];
       const int last = cap_of(j) - (j.fp32_phase ? 1 : 0);
-      if (j.stress_mask || j.n_eval + 1 >= last) continue;
+      if ((j.stress_mask && !j.fp32_phase) || j.n_eval + 1 >= last) continue;
       j.ahead = true;
       list.at[cnt++] = (uint8_t)q;
     }
