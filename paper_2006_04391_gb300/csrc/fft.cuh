@@ -304,16 +304,20 @@ __global__ void __launch_bounds__(Shape<T, N>::LP* Shape<T, N>::TPL)
     for (int k1 = 0; k1 < S::R1; ++k1) s[k1 * S::PITCH + t] = a[k1];
   }
   __syncthreads();
+  // (second stage: R1 threads a line, whole warps of them)
+  const int t2 = threadIdx.x % S::R1, l2 = threadIdx.x / S::R1;
+  const bool ok2 = l2 < S::LP && p - l + l2 < pairs;
+  cx<T>* s2 = reinterpret_cast<cx<T>*>(smem_) + l2 * S::ZLINE;
   cx<T> b[S::R2];
-  if (ok && t < S::R1) {
+  if (ok2) {
 #pragma unroll
-    for (int n2 = 0; n2 < S::R2; ++n2) b[n2] = s[t * S::PITCH + n2];
+    for (int n2 = 0; n2 < S::R2; ++n2) b[n2] = s2[t2 * S::PITCH + n2];
     Dft<S::R2, false, T>::run(b);
   }
   __syncthreads();
-  if (ok && t < S::R1) {
+  if (ok2) {
 #pragma unroll
-    for (int k2 = 0; k2 < S::R2; ++k2) s[t + S::R1 * k2] = b[k2];
+    for (int k2 = 0; k2 < S::R2; ++k2) s2[t2 + S::R1 * k2] = b[k2];
   }
   __syncthreads();
   if (ok) {
@@ -369,16 +373,19 @@ __global__ void __launch_bounds__(Shape<T, N>::LP* Shape<T, N>::TPL)
     }
   }
   __syncthreads();
+  const int t2 = threadIdx.x % S::R1, l2 = threadIdx.x / S::R1;
+  const bool ok2 = l2 < S::LP && p - l + l2 < pairs;
+  cx<T>* s2 = reinterpret_cast<cx<T>*>(smem_) + l2 * S::ZLINE;
   cx<T> b[S::R2];
-  if (ok && t < S::R1) {
+  if (ok2) {
 #pragma unroll
-    for (int k2 = 0; k2 < S::R2; ++k2) b[k2] = s[t + S::R1 * k2];
-    line_inv1<T, N>(b, t, tw);
+    for (int k2 = 0; k2 < S::R2; ++k2) b[k2] = s2[t2 + S::R1 * k2];
+    line_inv1<T, N>(b, t2, tw);
   }
   __syncthreads();
-  if (ok && t < S::R1) {
+  if (ok2) {
 #pragma unroll
-    for (int n2 = 0; n2 < S::R2; ++n2) s[t * S::PITCH + n2] = b[n2];
+    for (int n2 = 0; n2 < S::R2; ++n2) s2[t2 * S::PITCH + n2] = b[n2];
   }
   __syncthreads();
   if (ok) {
@@ -722,6 +729,15 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
   const int col = tile * S::GW + w;
   const bool ok = threadIdx.x < S::GL && col < cols;
   cx<T>* hat = static_cast<cx<T>*>(v.sig_hat) + col;
+  // this tile's share of the material kernel's partial sums, so that the job's
+  // last block has 7 sums of `tiles` left (256^3: 29 k values, not 102 k)
+  if (v.arrived && threadIdx.x < 6) {
+    const double* m = v.mat_part + (int64_t)threadIdx.x * v.n_vch;
+    const int k1 = (int)((int64_t)(tile + 1) * v.n_vch / tiles);
+    double sum = 0.0;
+    for (int k = (int)((int64_t)tile * v.n_vch / tiles); k < k1; ++k) sum += __ldg(m + k);
+    v.gam_part[(int64_t)(1 + threadIdx.x) * tiles + tile] = sum;
+  }
 #pragma unroll
   for (int c = c0; c < 6; c += S::CG) {
     if (!ok) break;
@@ -735,16 +751,19 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
     for (int k1 = 0; k1 < S::R1; ++k1) s[(k1 * S::PITCH + t) * S::GW] = a[k1];
   }
   __syncthreads();
+  // (the stages of R1 threads a line: whole warps of them)
+  const int t2 = (threadIdx.x / S::GW) % S::R1, d0 = threadIdx.x / (S::GW * S::R1);
+  const bool ok2 = d0 < S::CG && col < cols;
 #pragma unroll
-  for (int c = c0; c < 6; c += S::CG) {
-    if (!ok || t >= S::R1) break;
+  for (int c = d0; c < 6; c += S::CG) {
+    if (!ok2) break;
     cx<T>* s = sm + c * CS + w;
     cx<T> b[S::R2];
 #pragma unroll
-    for (int n2 = 0; n2 < S::R2; ++n2) b[n2] = s[(t * S::PITCH + n2) * S::GW];
+    for (int n2 = 0; n2 < S::R2; ++n2) b[n2] = s[(t2 * S::PITCH + n2) * S::GW];
     Dft<S::R2, false, T>::run(b);
 #pragma unroll
-    for (int k2 = 0; k2 < S::R2; ++k2) s[(t * S::PITCH + k2) * S::GW] = b[k2];
+    for (int k2 = 0; k2 < S::R2; ++k2) s[(t2 * S::PITCH + k2) * S::GW] = b[k2];
   }
   __syncthreads();
   double res[1] = {0.0};
@@ -774,15 +793,15 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
   res[0] *= 0.25;  // (s is 2 sig_hat)
   block_sum_at<1>(res, v.gam_part, tiles, tile);  // ends with a barrier
 #pragma unroll
-  for (int c = c0; c < 6; c += S::CG) {
-    if (!ok || t >= S::R1) break;
+  for (int c = d0; c < 6; c += S::CG) {
+    if (!ok2) break;
     cx<T>* s = sm + c * CS + w;
     cx<T> b[S::R2];
 #pragma unroll
-    for (int k2 = 0; k2 < S::R2; ++k2) b[k2] = s[(t * S::PITCH + k2) * S::GW];
-    line_inv1<T, N>(b, t, tw);
+    for (int k2 = 0; k2 < S::R2; ++k2) b[k2] = s[(t2 * S::PITCH + k2) * S::GW];
+    line_inv1<T, N>(b, t2, tw);
 #pragma unroll
-    for (int n2 = 0; n2 < S::R2; ++n2) s[(t * S::PITCH + n2) * S::GW] = b[n2];
+    for (int n2 = 0; n2 < S::R2; ++n2) s[(t2 * S::PITCH + n2) * S::GW] = b[n2];
   }
   __syncthreads();
 #pragma unroll
@@ -797,18 +816,19 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
 #pragma unroll
     for (int n1 = 0; n1 < S::R1; ++n1) hat_st(x + (int64_t)(n1 * S::R2 + t) * cols, a[n1]);
   }
-  // the job's last block forms its final sums (the material partials are those
-  // of the launch before)
+  // the job's last block forms its final sums
   if (v.arrived) {
     __shared__ bool last;
+    if (threadIdx.x < 6) __threadfence();  // this block's partials (written by these threads) before its arrival
+    __syncthreads();
     if (threadIdx.x == 0) {
-      __threadfence();  // this block's partial (written by this thread) before its arrival
+      __threadfence();
       last = atomicAdd(v.arrived, 1u) == (unsigned)tiles - 1u;
     }
     __syncthreads();
     if (last) {
       __threadfence();
-      finalize_sums(v.mat_part, v.n_vch, v.gam_part, tiles, v.inv_n3, v.mu0 * 1e-6, v.red, v.mean);
+      finalize_sums(v.gam_part + tiles, tiles, v.gam_part, tiles, v.inv_n3, v.mu0 * 1e-6, v.red, v.mean);
       if (threadIdx.x == 0) *v.arrived = 0u;
     }
   }

@@ -67,7 +67,7 @@ struct JobView {
   void* sig_hat;         // [6][nmodes]
   void* eps_hat;         // [6][nmodes]
   double* mat_part;      // [6][n_vch]
-  double* gam_part;      // [n_mch]
+  double* gam_part;      // [n_mch]; fused Green pass: [7][tiles], the error and the six stress sums
   double* mean;          // [6] the mean stress of the job's last evaluation (device)
   double E[6];           // mean strain
   Reduced* red;          // where the job's error and mean stress go (page-locked host memory)
@@ -399,8 +399,10 @@ __device__ __forceinline__ int owner(const int64_t* starts, int n, int64_t c) {
 }
 
 // Batched material evaluation: all jobs of the launch, chunk by chunk.
+// (FP32: 40 registers, twelve blocks an SM, 24 bytes spilled; the kernel waits on
+// loads: 256^3 385 us at nine blocks, 306 at ten, 300 at twelve, 346 at sixteen)
 template <class T, int MODE>
-__global__ void __launch_bounds__(kMatBlock) ms_material_batch_kernel(const JobView* __restrict__ views, int n_jobs,
+__global__ void __launch_bounds__(kMatBlock, MODE == MODE_FP32 ? 12 : 1) ms_material_batch_kernel(const JobView* __restrict__ views, int n_jobs,
                                                                       int64_t total_chunks) {
   __shared__ int64_t starts[kMaxBatch];
   __shared__ LawTable law;

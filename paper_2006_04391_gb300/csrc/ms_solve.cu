@@ -81,7 +81,7 @@ int64_t n_mchunks(int64_t nmodes) { return (nmodes + kMChunk - 1) / kMChunk; }
 int64_t n_gam_part(int N) {
   int64_t n = n_mchunks((int64_t)N * N * (N / 2 + 1));
   for (const FftOps* o : {fft_ops_f32(N), fft_ops_f64(N)})
-    if (o) n = std::max<int64_t>(n, o->green_tiles);
+    if (o) n = std::max<int64_t>(n, 7 * (int64_t)o->green_tiles);
   return n;
 }
 
