@@ -729,15 +729,6 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
   const int col = tile * S::GW + w;
   const bool ok = threadIdx.x < S::GL && col < cols;
   cx<T>* hat = static_cast<cx<T>*>(v.sig_hat) + col;
-  // this tile's share of the material kernel's partial sums, so that the job's
-  // last block has 7 sums of `tiles` left (256^3: 29 k values, not 102 k)
-  if (v.arrived && threadIdx.x < 6) {
-    const double* m = v.mat_part + (int64_t)threadIdx.x * v.n_vch;
-    const int k1 = (int)((int64_t)(tile + 1) * v.n_vch / tiles);
-    double sum = 0.0;
-    for (int k = (int)((int64_t)tile * v.n_vch / tiles); k < k1; ++k) sum += __ldg(m + k);
-    v.gam_part[(int64_t)(1 + threadIdx.x) * tiles + tile] = sum;
-  }
 #pragma unroll
   for (int c = c0; c < 6; c += S::CG) {
     if (!ok) break;
@@ -751,6 +742,19 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
     for (int k1 = 0; k1 < S::R1; ++k1) s[(k1 * S::PITCH + t) * S::GW] = a[k1];
   }
   __syncthreads();
+  // FP32 (bound by latency): the strain spectrum of a thread's next mode is
+  // loaded one mode ahead, the first during the second stage
+  constexpr bool kAhead = sizeof(T) == 4;
+  const bool project = v.project != 0;
+  cx<T>* eh = static_cast<cx<T>*>(v.eps_hat);
+  auto load_e = [&](int m, cx<T> (&e)[6]) {
+    const int mc = tile * S::GW + m % S::GW;
+    const bool in = m < N * S::GW && mc < cols && !project;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) e[q] = in ? hat_ld(eh + (int64_t)(m / S::GW) * cols + mc + q * modes) : cx<T>{T(0), T(0)};
+  };
+  cx<T> en[kAhead ? 6 : 1];
+  if constexpr (kAhead) load_e(threadIdx.x, en);
   // (the stages of R1 threads a line: whole warps of them)
   const int t2 = (threadIdx.x / S::GW) % S::R1, d0 = threadIdx.x / (S::GW * S::R1);
   const bool ok2 = d0 < S::CG && col < cols;
@@ -769,17 +773,22 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
   double res[1] = {0.0};
   {
     const T inv4mu = (T)v.inv4mu, coef = (T)v.green_b;
-    const bool project = v.project != 0;
-    cx<T>* eh = static_cast<cx<T>*>(v.eps_hat);
     for (int m = threadIdx.x; m < N * S::GW; m += S::GT) {
       const int mw = m % S::GW, kx = m / S::GW;
       const int mc = tile * S::GW + mw;
+      cx<T> sg[6], e[6];
+      if constexpr (kAhead) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) e[q] = en[q];
+        load_e(m + S::GT, en);
+      }
       if (mc >= cols) continue;
       cx<T>* g = eh + (int64_t)kx * cols + mc;
-      cx<T>* sl = sm + ((kx % S::R1) * S::PITCH + kx / S::R1) * S::GW + mw;
-      cx<T> sg[6], e[6];
+      if constexpr (!kAhead) {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) e[q] = project ? cx<T>{T(0), T(0)} : hat_ld(g + q * modes);
+        for (int q = 0; q < 6; ++q) e[q] = project ? cx<T>{T(0), T(0)} : hat_ld(g + q * modes);
+      }
+      cx<T>* sl = sm + ((kx % S::R1) * S::PITCH + kx / S::R1) * S::GW + mw;
 #pragma unroll
       for (int q = 0; q < 6; ++q) sg[q] = sl[q * CS];
       green_mode<T, N>(kx, mc / S::Nh, mc % S::Nh, inv4mu, coef, sg, e, res[0]);
@@ -792,6 +801,17 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
   }
   res[0] *= 0.25;  // (s is 2 sig_hat)
   block_sum_at<1>(res, v.gam_part, tiles, tile);  // ends with a barrier
+  // this tile's share of the material kernel's partial sums, so that the job's
+  // last block has 7 sums of `tiles` left (256^3: 29 k values, not 102 k); here,
+  // where the fence overlaps the other warps' inverse transform
+  if (v.arrived && threadIdx.x < 6) {
+    const double* m = v.mat_part + (int64_t)threadIdx.x * v.n_vch;
+    const int k1 = (int)((int64_t)(tile + 1) * v.n_vch / tiles);
+    double sum = 0.0;
+    for (int k = (int)((int64_t)tile * v.n_vch / tiles); k < k1; ++k) sum += __ldg(m + k);
+    v.gam_part[(int64_t)(1 + threadIdx.x) * tiles + tile] = sum;
+    __threadfence();  // the block's partials (this thread's and, thread 0, the error's) before its arrival
+  }
 #pragma unroll
   for (int c = d0; c < 6; c += S::CG) {
     if (!ok2) break;
@@ -804,6 +824,11 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
     for (int n2 = 0; n2 < S::R2; ++n2) s[(t2 * S::PITCH + n2) * S::GW] = b[n2];
   }
   __syncthreads();
+  __shared__ bool last;
+  if (v.arrived && threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(v.arrived, 1u) == (unsigned)tiles - 1u;
+  }
 #pragma unroll
   for (int c = c0; c < 6; c += S::CG) {
     if (!ok) break;
@@ -818,13 +843,6 @@ __global__ void __launch_bounds__(Shape<T, N>::GT)
   }
   // the job's last block forms its final sums
   if (v.arrived) {
-    __shared__ bool last;
-    if (threadIdx.x < 6) __threadfence();  // this block's partials (written by these threads) before its arrival
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      last = atomicAdd(v.arrived, 1u) == (unsigned)tiles - 1u;
-    }
     __syncthreads();
     if (last) {
       __threadfence();
