@@ -40,12 +40,11 @@ constexpr int kOdeBlock = 128;
 // 3645 us with 1, 3502 with 4, 3686 with 8, 4108 with 12.
 constexpr int kRefill = 4;
 
-// Per-lane scheduling (without the tangent): a lane takes voxels i, i +
-// stride, ... and starts its next voxel as soon as the current one has
-// finished its substeps; the warp runs while any lane has work.  Voxels need
-// different substep counts, and with one voxel per lane per pass the finished
-// lanes would idle until the slowest voxel of their warp is done (measured:
-// 23.7 of 32 lanes busy; 28.7 -> 31.2 M voxel-updates/s).
+// Per-lane scheduling (without the tangent): a lane starts its next voxel when
+// its current one has finished its substeps; the warp runs while any lane has
+// work.  Voxels need different substep counts, and with one voxel per lane per
+// pass the finished lanes would idle until the slowest voxel of their warp is
+// done.
 template <class Law, bool TAN, int PAIR>
 __global__ void __launch_bounds__(kOdeBlock) ode23_kernel(int64_t n, int64_t ld, LawParams<double> p, Step hs,
                                                           Ode23Ctl ctl, const double* __restrict__ epsn,
@@ -100,7 +99,16 @@ __global__ void __launch_bounds__(kOdeBlock) ode23_kernel(int64_t n, int64_t ld,
     }
     return;
   }
-  bool have = i < n;
+  // a block owns a contiguous range of voxels; its lanes take the next one of it
+  // from a shared counter, so they finish together whatever their substep counts
+  // (200 k voxels: 3502 -> 3174 us against a fixed stride per lane)
+  const int64_t per = (n + gridDim.x - 1) / gridDim.x, first = (int64_t)blockIdx.x * per;
+  const int64_t last = first + per < n ? first + per : n;
+  __shared__ unsigned long long taken;
+  if (threadIdx.x == 0) taken = blockDim.x;
+  __syncthreads();
+  i = first + threadIdx.x;
+  bool have = i < last;
   if (have) start(i);
   for (;;) {
     const bool busy = have && !v.done;
@@ -117,8 +125,8 @@ __global__ void __launch_bounds__(kOdeBlock) ode23_kernel(int64_t n, int64_t ld,
 #pragma unroll
         for (int c = 0; c < NZ; ++c) z[c * ld + i] = zo[c];
         if (status) status[i] = (int32_t)st;
-        i += stride;
-        have = i < n;
+        i = first + (int64_t)atomicAdd(&taken, 1ull);
+        have = i < last;
         if (have) start(i);
       }
     }

@@ -17,7 +17,8 @@
 // Bound: the FP64 pipe.  The AD sweeps of ode23.cuh took about 800 FP64
 // operations an attempt; this takes about 200 (odd integer n: Q^(b_Psi - 1) is
 // a product of Q) or 290 (else: the table power).  Measured on 200 k voxels, n =
-// 5, rtol 1e-3: 7568 -> 3502 us.
+// 5, rtol 1e-3: 7568 -> 3502 us, 3174 with the voxels of a block taken from a
+// shared counter (ode_kernel.cuh).
 #pragma once
 
 // (included by ode23.cuh)
