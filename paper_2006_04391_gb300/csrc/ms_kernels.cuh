@@ -56,7 +56,7 @@ struct Reduced {
 
 // One job of a batched launch (device copy, rebuilt by the host every tick).
 struct JobView {
-  RayConst ray[kMaxPhases];  // the scalar equation of each Norton phase at this step's h
+  RayConst ray[kMaxPhases];  // the scalar equation of each phase at this step's h (elastic: its moduli)
   int kind[kMaxPhases];      // GSM_PSI_* of each phase
   const uint8_t* phase;
   const void* eps_raw;   // [6][nvox] N^3 * strain (inverse transform's output); FP32 fields: without its mean
@@ -182,14 +182,16 @@ struct LawTable {
 // 1/N^3 scaling and of the lane's partial stress sums (FP32 fields: no FP64
 // work, a sixty-fourth of the FP32 rate on GB300; the block sums are FP64).
 // All loads are issued before the phase is known: z_n of an elastic voxel is
-// read for nothing, but no load waits for another.
+// read for nothing, but no load waits for another.  An elastic voxel is the
+// Norton voxel that does not flow (theta = 0, t = 1, z = 0): one instruction
+// stream for both, where a branch cost the warps that hold both kinds both.
 template <class T, int MODE>
 __device__ __forceinline__ void material_voxel(int64_t i, int64_t nvox, const uint8_t* __restrict__ phase,
-                                               const PhaseTable& tab, const LawTable& law, T inv_n3,
+                                               const LawTable& law, T inv_n3,
                                                const T* __restrict__ eps_raw, const T* __restrict__ zn,
                                                T* __restrict__ sig, T* __restrict__ z, T (&acc)[6]) {
   const int ph = (int)__ldg(phase + i);
-  T e[6], zi[6], s[6], zo[6] = {0, 0, 0, 0, 0, 0};
+  T e[6], zi[6], s[6], zo[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) e[c] = __ldg(eps_raw + c * nvox + i);
 #pragma unroll
@@ -199,12 +201,11 @@ __device__ __forceinline__ void material_voxel(int64_t i, int64_t nvox, const ui
     if constexpr (sizeof(T) == 4) e[c] = fmaf(e[c], inv_n3, law.E_lo[c]) + law.E_hi[c];
     else e[c] *= inv_n3;
   }
-  if (law.kind[ph] == GSM_PSI_ELASTIC_VP_DEV) {
-    voxel_ray<NortonDev>(law.ray[ph], e, zi, true, MODE == MODE_FP32_FIX, s, zo, static_cast<T*>(nullptr));
-  } else {
-    if constexpr (sizeof(T) == 8) voxel_elastic<double>(tab.p64[ph], e, s, nullptr);
-    else voxel_elastic<float>(tab.p32[ph], e, s, nullptr);
-  }
+  const bool vp = law.kind[ph] == GSM_PSI_ELASTIC_VP_DEV;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) zi[c] = vp ? zi[c] : T(0);
+  voxel_ray<NortonDev>(law.ray[ph], e, zi, vp, MODE == MODE_FP32_FIX, s, zo, static_cast<T*>(nullptr));
+  zo[2] = vp ? zo[2] : T(0);
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
     if constexpr (sizeof(T) == 4) sig[c * nvox + i] = s[c] - law.sub[c];
@@ -375,13 +376,13 @@ __global__ void __launch_bounds__(kMatBlock) ms_material_kernel(int64_t nvox, co
   __shared__ LawTable law;
   if (threadIdx.x < kMaxPhases) {
     law.kind[threadIdx.x] = tab.kind[threadIdx.x];
-    if (tab.kind[threadIdx.x] == GSM_PSI_ELASTIC_VP_DEV) law.ray[threadIdx.x] = make_ray(tab.p64[threadIdx.x], h);
+    law.ray[threadIdx.x] = make_ray(tab.p64[threadIdx.x], h);
   }
   __syncthreads();
   T acc[6] = {0, 0, 0, 0, 0, 0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += stride)
-    material_voxel<T, MODE>(i, nvox, phase, tab, law, (T)inv_n3, eps_raw, zn, sig, z, acc);
+    material_voxel<T, MODE>(i, nvox, phase, law, (T)inv_n3, eps_raw, zn, sig, z, acc);
   double accd[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) accd[c] = (double)acc[c];
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(kMatBlock, MODE == MODE_FP32 ? 12 : 1) ms_mate
     for (int o = threadIdx.x; o < v.chunk; o += kMatBlock) {
       const int64_t i = lc * v.chunk + o;
       if (i < v.nvox)
-        material_voxel<T, MODE>(i, v.nvox, v.phase, *v.tab, law, (T)v.inv_n3, static_cast<const T*>(v.eps_raw),
+        material_voxel<T, MODE>(i, v.nvox, v.phase, law, (T)v.inv_n3, static_cast<const T*>(v.eps_raw),
                                 static_cast<const T*>(v.zn), static_cast<T*>(v.sig), static_cast<T*>(v.z), acc);
     }
     double accd[6];

@@ -644,7 +644,7 @@ int step_start(Engine& g, Job& j) {
   }
   mixed_setup(j);
   for (int p = 0; p < j.n_phases; ++p)
-    if (j.tab_host.kind[p] == GSM_PSI_ELASTIC_VP_DEV) j.ray[p] = make_ray(j.tab_host.p64[p], j.h[j.step]);
+    if (j.tab_host.kind[p] != GSM_PSI_ELASTIC_VP_KIN) j.ray[p] = make_ray(j.tab_host.p64[p], j.h[j.step]);
   j.n_eval = 0;
   j.n32 = 0;
   j.best = 1e300;
