@@ -52,26 +52,30 @@ ALG_POWS = {"predictor": 0, "line": 3, "newton": 3, "residual": 1, "subst": 0, "
 # FP64 refinement step of 12 flops, a power and an exponential.
 MODEL_FLOPS, MODEL_POWS = 9, 2
 MODEL64_FLOPS, MODEL64_POWS = 12, 2
+# The Norton law's step has its root on the predictor segment, and the GPU
+# solves it there: status words without a Newton iteration (FP64 corrections
+# apart).  Hand count of that scalar form: trial strain 13, its norm 12, one
+# evaluation with its Halley step 19 and a power, stress and internal variables 23.
+RAY_FLOPS = {"trial": 13, "norm": 12, "eval": 19, "result": 23}
 #
 # * executed FP64 operations: each DADD, DMUL or DFMA takes one FP64 issue
 #   slot and GB300 issues two FP64 operations per SM per cycle (ncu
 #   peak_sustained).  Operations per voxel, counted by ncu
 #   (smsp__sass_thread_inst_executed_op_{dadd,dmul,dfma}_pred_on) on this
 #   workload at three step sizes (profiles/norton_kernel_fp64_op_counts_2p20.md):
-#     FP32 bulk + correction (double-float residual and power): 50.52 per
+#     FP32 bulk + correction (double-float residual and power): 33.15 per
 #       voxel with one correction; a further correction repeats the power's
 #       FP64 exponent product and the conversions (~5, estimated; one
 #       correction is the rule);
-#     FP64: 806.5 per voxel at the two line-search evaluations every voxel
-#       takes since the search starts from the segment model's root; 158.8 per
-#       further evaluation (the earlier fit over three step sizes).
+#     FP64: 74.05 per voxel with one evaluation (42 of them the evaluation: the
+#       power 27, the Halley step and the residual).
 #   They explain the gap between the algorithmic rate and the peak: a power
 #   (one algorithmic operation) executes as tens of FP64 operations.
 FP64_ISSUE_PER_SM_CLK = 2
-OPS_FIX_FIRST = 50.52
+OPS_FIX_FIRST = 33.15
 OPS_FIX_EXTRA = 5.0
-OPS_FP64_BASE = 488.9
-OPS_FP64_LINE = 158.8
+OPS_FP64_BASE = 32.05
+OPS_FP64_LINE = 42.0
 BYTES_PER_VOXEL_FP64 = 4 * 6 * 8          # eps, z_n in; sigma, z out
 # DRAM bytes of one full-size FP32-bulk launch (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum, one capture of launch 6 of this workload: the
@@ -257,13 +261,19 @@ def alg_flops_per_voxel(status, mode):
     Newton step) + stress, all FP64.  FP32 bulk + FP64 correction: the
     predictor, search and Newton steps of the FP32 solve are FP32; each FP64
     correction is an FP64 residual sweep, substitutions with the FP32 factor
-    (FP32) and w += dw (5 FP64 adds); the stress is FP64."""
+    (FP32) and w += dw (5 FP64 adds); the stress is FP64.  A voxel solved on the
+    predictor segment (no Newton iteration) counts RAY_FLOPS instead."""
+    import numpy as np
     line, newton, fix, model = _status_fields(status, model=True)
-    A, W = ALG_FLOPS, ALG_POWS
+    A, W, R = ALG_FLOPS, ALG_POWS, RAY_FLOPS
+    ray = newton - fix == 0
+    evals = fix if mode != "fp64" else line
+    ray_f = R["trial"] + R["norm"] + R["eval"] * evals + R["result"]
     if mode == "fp64":
         step64 = model > 0
         f64 = A["predictor"] + A["line"] * line + A["newton"] * newton + A["stress"] + MODEL64_FLOPS * step64
         p64 = W["line"] * line + W["newton"] * newton + MODEL64_POWS * step64
+        f64, p64 = np.where(ray, ray_f, f64), np.where(ray, evals, p64)
         return float(f64.mean()), float((MODEL_FLOPS * model).mean()), float(p64.mean()), \
             float((MODEL_POWS * model).mean())
     bulk = newton - fix
@@ -271,6 +281,9 @@ def alg_flops_per_voxel(status, mode):
     p32 = W["line"] * line + W["newton"] * bulk + MODEL_POWS * model
     f64 = (A["residual"] + 5) * fix + A["stress"]
     p64 = W["residual"] * fix
+    f32 = np.where(ray, MODEL_FLOPS * model, f32)
+    p32 = np.where(ray, MODEL_POWS * model, p32)
+    f64, p64 = np.where(ray, ray_f, f64), np.where(ray, evals, p64)
     return float(f64.mean()), float(f32.mean()), float(p64.mean()), float(p32.mean())
 
 
