@@ -527,9 +527,9 @@ def report(args, world, rank, results, e2e_ms, ms_block, serve_block=None, adj_b
                      "alg_fp64_flops_per_voxel": a32_64, "alg_fp64_pow_per_voxel": pw32_64,
                      "alg_fp32_flops_per_voxel": a32_32, "alg_fp32_pow_per_voxel": pw32_32,
                      "fp32_achieved": ach32, "fp32_peak": P32, "fp32_frac": ach32 / P32,
-                     "note": "achieved = algorithmic FP64 flops of the FP64 corrections and the stress (oracle "
-                             "counts x the kernel's iteration counts; pow counted apart) / mean launch time; the FP32 "
-                             "solve runs on the FP32 pipe (fp32_*)",
+                     "note": "achieved = algorithmic FP64 flops of the scalar equation's correction and the results "
+                             "(trial strain, norm, one evaluation, results; pow counted apart) / mean launch time; "
+                             "the FP32 solve runs on the FP32 pipe (fp32_*)",
                      "executed_fp64_ops_per_voxel": fpv32,
                      "issue_frac": fpv32 * N_VOX / t32 / 1e9 / issue_peak,
                      "hbm_frac": BYTES_PER_VOXEL_FP64 * N_VOX / t32 / 1e9 / peaks.get("hbm_gbs", 6783.1)},
