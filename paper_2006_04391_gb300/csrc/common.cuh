@@ -30,6 +30,7 @@ inline LawParams<double> make_params(const double* prm, int kind) {
   p.H_kin = 0.0;
   p.sig_Y = 0.0;
   p.L_ode = 0.0;
+  p.q_ode = 0.0;
   if (kind == 2) {
     const double sY = prm[2], H = prm[3], e0 = prm[4], sd = prm[5], n = prm[6];
     p.a_phi = 1.0;
@@ -44,7 +45,8 @@ inline LawParams<double> make_params(const double* prm, int kind) {
     p.c_phi = s0 * e0 * n / (n + 1.0) * std::pow(e0, -(n + 1.0) / n);
     p.b_Psi = (n + 1.0) / 2.0;
     p.c_Psi = s0 * e0 / (n + 1.0) * std::pow(s0, -(n + 1.0));
-    p.L_ode = 6.0 * p.mu * p.c_Psi * p.b_Psi * std::pow(12.0 * p.mu * p.mu, p.b_Psi - 1.0);
+    p.L_ode = 3.0 * p.mu * e0 / s0;
+    p.q_ode = 12.0 * (p.mu / s0) * (p.mu / s0);
   } else {
     p.a_phi = 1.0;
     p.c_phi = 0.0;
@@ -65,6 +67,7 @@ inline LawParams<float> to_float(const LawParams<double>& p) {
   q.H_kin = (float)p.H_kin;
   q.sig_Y = (float)p.sig_Y;
   q.L_ode = (float)p.L_ode;
+  q.q_ode = (float)p.q_ode;
   return q;
 }
 

@@ -31,7 +31,8 @@ template <class T> struct LawParams {
   T b_Psi;
   T H_kin;        // kinematic hardening modulus H (MichelSuquet)
   T sig_Y;        // yield stress, K(alpha) = sigma_Y (MichelSuquet)
-  T L_ode;        // flow factor 6 mu c_Psi b_Psi (12 mu^2)^(b_Psi - 1) (NortonDev, ode_ray.cuh)
+  T L_ode;        // flow factor 3 mu edot0 / sigma0 (NortonDev, ode_ray.cuh)
+  T q_ode;        // 12 mu^2 / sigma0^2
 };
 
 // Linear elasticity: psi = 1/2 eps^T C eps, no internal variables.

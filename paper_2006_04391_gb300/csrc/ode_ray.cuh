@@ -4,8 +4,12 @@
 // With psi isotropic and Psi = c_Psi (s_A^2)^b_Psi, s_A the von Mises norm of
 // A = -psi_y, the flow is ydot = Lambda x with x the y-components of
 // dev(eps) - P y and
-//   Lambda = 6 mu c_Psi b_Psi (12 mu^2 Q)^(b_Psi - 1) = L_ode Q^(b_Psi - 1),
-//   Q = x0^2 + x1^2 + x0 x1 + (x2^2 + x3^2 + x4^2)/4     (s_A^2 = 12 mu^2 Q).
+//   Lambda = 6 mu c_Psi b_Psi (12 mu^2 Q)^(b_Psi - 1) = L_ode (q_ode Q)^(b_Psi - 1),
+//   Q = x0^2 + x1^2 + x0 x1 + (x2^2 + x3^2 + x4^2)/4     (s_A^2 = 12 mu^2 Q),
+//   L_ode = 3 mu edot0 / sigma0,  q_ode = 12 mu^2 / sigma0^2:
+// the power's base is (s_A / sigma0)^2, of order one wherever the law flows, so
+// neither the base nor the factor leaves the FP64 range, whatever the units and
+// the exponent (as one number, (12 mu^2)^(b_Psi - 1) overflows for E in Pa at n = 28).
 // The strain is linear over the step, so x obeys the autonomous equation
 //   xdot = edot - Lambda(x) x,
 // and a Runge-Kutta method applied to x is the one applied to y (affine
@@ -43,7 +47,8 @@ template <class Law, int PAIR> struct RayErkVoxel {
   bool last_rejected, done;
 
   AD_HD static double lambda(const LawParams<double>& p, const double (&v)[5]) {
-    const double Q = fma(v[0], v[0] + v[1], v[1] * v[1]) + 0.25 * fma(v[4], v[4], fma(v[3], v[3], v[2] * v[2]));
+    const double Q =
+        p.q_ode * (fma(v[0], v[0] + v[1], v[1] * v[1]) + 0.25 * fma(v[4], v[4], fma(v[3], v[3], v[2] * v[2])));
     // b_Psi - 1 a small integer, from the bits (the same for every lane; an FP64
     // compare or conversion would occupy the FP64 pipe)
     const uint64_t b = fpow::bits_of(p.b_Psi);
