@@ -61,14 +61,14 @@ struct JobView {
   const uint8_t* phase;
   const void* eps_raw;   // [6][nvox] N^3 * strain (inverse transform's output); FP32 fields: without its mean
   const void* zn;        // [6][nvox]
-  void* sig;             // [6][nvox] stress; FP32 fields: less the mean stress of the evaluation before
+  void* sig;             // [6][nvox] stress; FP32 fields: less *mean
   void* eps_out;         // [6][nvox] where the inverse transform writes the next strain
   void* z;               // [6][nvox]
   void* sig_hat;         // [6][nmodes]
   void* eps_hat;         // [6][nmodes]
   double* mat_part;      // [6][n_vch]
   double* gam_part;      // [n_mch]; fused Green pass: [7][tiles], the error and the six stress sums
-  double* mean;          // [6] the mean stress of the job's last evaluation (device)
+  double* mean;          // [6] the mean stress of the step's last evaluation, 0 at its first (device)
   double E[6];           // mean strain
   Reduced* red;          // where the job's error and mean stress go (page-locked host memory)
   unsigned* arrived;     // blocks of the fused Green pass that are done (0 between launches), or NULL
@@ -169,9 +169,9 @@ __device__ __forceinline__ void block_sum6_at(const double (&v)[6], double* out,
 //
 // FP32 fields hold what varies: the strain without its mean E (added here as a
 // pair of FP32 numbers) and the stress less a uniform one (the mean of the
-// evaluation before; the Green operator does not see the zero mode).  Their
-// rounding, and that of the transforms, is then relative to the fluctuations
-// and not to the means.
+// evaluation before, zero at a step's first; the Green operator does not see the
+// zero mode).  Their rounding, and that of the transforms, is then relative to
+// the fluctuations and not to the means.
 struct LawTable {
   RayConst ray[kMaxPhases];
   int kind[kMaxPhases];

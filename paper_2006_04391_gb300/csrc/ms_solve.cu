@@ -651,6 +651,9 @@ int step_start(Engine& g, Job& j) {
   j.since_best = 0;
   j.fp32_phase = j.precision == MS_PREC_FP32_BULK && cap_of(j) > 1;
   if (j.fp32_phase) {
+    // the step's first evaluation subtracts nothing from its stress: a step depends
+    // on its strain, z_n and load alone, not on what the context ran before
+    cudaMemsetAsync(j.mean_dev, 0, 6 * sizeof(double), g.stream);
     double off[6];
     for (int q = 0; q < 6; ++q) off[q] = -(double)j.nvox * j.E_prev[q];
     offset_convert<double, float>(g.stream, j.f64.eps_raw, j.f32.eps_raw, j.nvox, off);
