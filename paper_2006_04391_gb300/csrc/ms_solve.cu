@@ -186,8 +186,11 @@ struct Engine {
           cudaGetLastError();
           return GSM_ENOMEM;
         }
-        if (cudaMemcpy(p.tw, fp32 ? (const void*)twf.data() : (const void*)tw.data(), bytes, cudaMemcpyHostToDevice) !=
-            cudaSuccess) {
+        // on the engine's stream, which need not wait for the legacy default one, and
+        // waited for: the tables above are pageable and end here
+        if (cudaMemcpyAsync(p.tw, fp32 ? (const void*)twf.data() : (const void*)tw.data(), bytes,
+                            cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+            cudaStreamSynchronize(stream) != cudaSuccess) {
           cudaFree(p.tw);
           return GSM_ECUDA;
         }
