@@ -16,13 +16,16 @@
 // change of variable; the stage abscissae equal the row sums).  The stresses
 // are sigma = kappa tr(eps) 1 + 2 mu x, and the pair's stress difference is
 // 2 mu times the embedded difference of x: no stress is evaluated twice and
-// the difference does not cancel.
+// the difference does not cancel.  y is carried beside x and takes the flow
+// Lambda x of the accepted substeps: as dev(eps) - x a flow that is small beside
+// the strain would be rounded to the strain's last place.
 //
 // Bound: the FP64 pipe.  The AD sweeps of ode23.cuh took about 800 FP64
 // operations an attempt; this takes about 200 (odd integer n: Q^(b_Psi - 1) is
 // a product of Q) or 290 (else: the table power).  Measured on 200 k voxels, n =
-// 5, rtol 1e-3: 7568 -> 3502 us, 3174 with the voxels of a block taken from a
-// shared counter (ode_kernel.cuh).
+// 5, rtol 1e-3: 7568 -> 3502 us, 3177 with the voxels of a block taken from a
+// shared counter (ode_kernel.cuh), the same with y beside x (the embedded
+// difference from edot - f and the end rates pays for it).
 #pragma once
 
 // (included by ode23.cuh)
@@ -38,7 +41,7 @@ AD_HD double absmax_bits(double a, double b) {
 
 template <class Law, int PAIR> struct RayErkVoxel {
   double x[5], k1[5], ed[5];  // elastic deviatoric strain, its rate, the strain rate
-  double e0[5], de[5];        // y-components of dev(eps_n) and of dev(eps_{n+1}) - dev(eps_n)
+  double y[5], L1;            // internal variables; Lambda at x
   double hyd0, dhyd;          // kappa tr(eps_n) and its increment
   double sig_old[6];
   double t, dt;
@@ -64,10 +67,12 @@ template <class Law, int PAIR> struct RayErkVoxel {
     }
     return p.L_ode * fpow::pow_pos(Q, p.b_Psi - 1.0);
   }
-  AD_HD void rate(const LawParams<double>& p, const double (&v)[5], double (&k)[5]) const {
+  // k = edot - Lambda v; returns Lambda
+  AD_HD double rate(const LawParams<double>& p, const double (&v)[5], double (&k)[5]) const {
     const double L = lambda(p, v);
 #pragma unroll
     for (int a = 0; a < 5; ++a) k[a] = fma(-L, v[a], ed[a]);
+    return L;
   }
   AD_HD void stress(const LawParams<double>& p, double hyd, const double (&v)[5], double (&s)[6]) const {
     const double m2 = p.mu + p.mu;
@@ -86,18 +91,20 @@ template <class Law, int PAIR> struct RayErkVoxel {
     double d[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) d[i] = e1_[i] - e0_[i];
-    const double dtr = d[0] + d[1] + d[2];
-    hyd0 = kappa * tr0;
-    dhyd = kappa * dtr;
-    const double yn[5] = {zn[0], zn[1], zn[3], zn[4], zn[5]};
+    // deviators from differences: a hydrostatic strain leaves no rounding in them
+    auto dev = [](const double (&e)[6], int a) {
+      return a < 2 ? ((e[a] - e[1 - a]) + (e[a] - e[2])) * (1.0 / 3.0) : e[a + 1];
+    };
+    // (0 times: a non-finite increment or z_n shows in the stress from the start)
 #pragma unroll
     for (int a = 0; a < 5; ++a) {
-      e0[a] = a < 2 ? fma(tr0, -1.0 / 3.0, e0_[a]) : e0_[a + 1];
-      de[a] = a < 2 ? fma(dtr, -1.0 / 3.0, d[a]) : d[a + 1];
-      ed[a] = de[a] * inv_h;
-      x[a] = e0[a] - yn[a];
+      ed[a] = dev(d, a) * inv_h;
+      y[a] = zn[a < 2 ? a : a + 1];
+      x[a] = fma(0.0, ed[a], dev(e0_, a) - y[a]);
     }
-    rate(p, x, k1);
+    dhyd = kappa * (d[0] + d[1] + d[2]);
+    hyd0 = fma(0.0, dhyd + (y[0] + y[1]), kappa * tr0);
+    L1 = rate(p, x, k1);
     stress(p, hyd0, x, sig_old);
     t = 0.0;
     dt = hs.h;
@@ -118,50 +125,52 @@ template <class Law, int PAIR> struct RayErkVoxel {
     if (clip) dt = h - t;
     const double tn1 = clip ? h : t + dt;
     const double th1 = clip ? 1.0 : tn1 * hs.inv_h;
-    double xn[5], e[5], k[5], v[5];
+    // f: the pair's flow, sum of b_i Lambda_i x_i; xn = x + dt (edot - f), y takes dt f;
+    // e: de times the embedded difference's rate
+    constexpr double de = PAIR == ERK_BS23 ? 0.25 : 0.5;
+    double xn[5], e[5], f[5], k[5], v[5], Ln;
     if constexpr (PAIR == ERK_BS23) {
       constexpr double b1 = 2.0 / 9.0, b2 = 1.0 / 3.0, b3 = 4.0 / 9.0;
-      constexpr double e1 = 2.0 / 9.0 - 7.0 / 24.0, e2 = 1.0 / 3.0 - 1.0 / 4.0, e3 = 4.0 / 9.0 - 1.0 / 3.0,
-                       e4 = -1.0 / 8.0;
-      const double c2 = 0.5 * dt, c3 = 0.75 * dt;
+      const double c2 = 0.5 * dt, c3 = 0.75 * dt, w1 = b1 * L1;
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
         v[a] = fma(c2, k1[a], x[a]);
-        xn[a] = b1 * k1[a];
-        e[a] = e1 * k1[a];
+        f[a] = w1 * x[a];
       }
-      rate(p, v, k);
+      const double w2 = b2 * rate(p, v, k);
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
+        f[a] = fma(w2, v[a], f[a]);
         v[a] = fma(c3, k[a], x[a]);
-        xn[a] = fma(b2, k[a], xn[a]);
-        e[a] = fma(e2, k[a], e[a]);
       }
-      rate(p, v, k);
+      const double w3 = b3 * rate(p, v, k);
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
-        xn[a] = fma(dt, fma(b3, k[a], xn[a]), x[a]);
-        e[a] = fma(e3, k[a], e[a]);
+        f[a] = fma(w3, v[a], f[a]);
+        e[a] = ed[a] - f[a];  // sum of b_i k_i
+        xn[a] = fma(dt, e[a], x[a]);
       }
-      rate(p, xn, k);  // k1 of the next substep
+      Ln = rate(p, xn, k);  // k1 of the next substep
+      // the difference of the two weights, (-5/72, 1/12, 1/9, -1/8), is 1/4 (b, 0) - 1/8 (1, 0, 0, 1)
 #pragma unroll
-      for (int a = 0; a < 5; ++a) e[a] = fma(e4, k[a], e[a]);
+      for (int a = 0; a < 5; ++a) e[a] = fma(-0.5, k1[a] + k[a], e[a]);
     } else {
       // Heun (order 2) continued, explicit Euler embedded: difference dt/2 (k2 - k1)
 #pragma unroll
       for (int a = 0; a < 5; ++a) v[a] = fma(dt, k1[a], x[a]);
-      rate(p, v, k);
+      const double w1 = 0.5 * L1, w2 = 0.5 * rate(p, v, k);
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
-        xn[a] = fma(0.5 * dt, k1[a] + k[a], x[a]);
-        e[a] = 0.5 * (k[a] - k1[a]);
+        f[a] = fma(w2, v[a], w1 * x[a]);
+        xn[a] = fma(dt, ed[a] - f[a], x[a]);
+        e[a] = k[a] - k1[a];
       }
-      rate(p, xn, k);
+      Ln = rate(p, xn, k);
     }
     double s[6];
     stress(p, fma(th1, dhyd, hyd0), xn, s);
     // stress difference of the pair (the hydrostatic parts are the same)
-    const double md = p.mu * dt, m2d = md + md;
+    const double md = p.mu * dt * de, m2d = md + md;
     const double d[6] = {m2d * e[0], m2d * e[1], -m2d * (e[0] + e[1]), md * e[2], md * e[3], md * e[4]};
     double sum = 0.0;
 #pragma unroll
@@ -169,15 +178,17 @@ template <class Law, int PAIR> struct RayErkVoxel {
     // err^2, err the RMS; a trial step that overflows is rejected like one with a large error
     const double err2 = finite64(sum) ? sum * (1.0 / 6.0) : 1e300;
     // 0.9 err^(-1/3) (ode23), 0.9 err^(-1/2) (ode12)
-    const double f = err2 == 0.0 ? 1e300 : 0.9 * fpow::pow_pos(err2, PAIR == ERK_BS23 ? -1.0 / 6.0 : -1.0 / 4.0);
-    const double grow = fmin(last_rejected ? 1.0 : 5.0, fmax(0.2, f));
+    const double fac = err2 == 0.0 ? 1e300 : 0.9 * fpow::pow_pos(err2, PAIR == ERK_BS23 ? -1.0 / 6.0 : -1.0 / 4.0);
+    const double grow = fmin(last_rejected ? 1.0 : 5.0, fmax(0.2, fac));
     if (err2 <= 1.0) {
       t = tn1;
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
+        y[a] = fma(dt, f[a], y[a]);
         x[a] = xn[a];
         k1[a] = k[a];
       }
+      L1 = Ln;
 #pragma unroll
       for (int i = 0; i < 6; ++i) sig_old[i] = s[i];
       ++n_acc;
@@ -193,10 +204,6 @@ template <class Law, int PAIR> struct RayErkVoxel {
   AD_HD unsigned finish(double h, double (&sig)[6], double (&z)[6], double*) const {
 #pragma unroll
     for (int i = 0; i < 6; ++i) sig[i] = sig_old[i];
-    const double th = t >= h ? 1.0 : t / h;
-    double y[5];
-#pragma unroll
-    for (int a = 0; a < 5; ++a) y[a] = fma(th, de[a], e0[a]) - x[a];
     z[0] = y[0];
     z[1] = y[1];
     z[2] = -(y[0] + y[1]);
