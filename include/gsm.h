@@ -32,12 +32,14 @@
  * Per-voxel status word (int32, optional output of gsm_update):
  *   bits 0-7 line-search iterations (evaluations of the segment function in the
  *   working precision), bits 8-15 Newton iterations (including FP64
- *   corrections), bit 16 converged, bit 17 non-finite input or result,
- *   bit 18 iteration cap reached, bit 19 Newton matrix not positive definite,
- *   bits 20-23 FP64 corrections (GSM_FP32_FP64FIX), bits 24-30 scalar
- *   iterations of the segment model that starts the line search.  The Norton
- *   law's step has its root on the predictor segment: it takes scalar iterations
- *   (FP32) and one evaluation there, no Newton iteration of the full system.
+ *   corrections), bit 16 converged (Norton law: not beside a trial strain that
+ *   is not finite), bit 17 non-finite input or result, bit 18 iteration cap
+ *   reached (or an iteration that left the range), bit 19 Newton matrix not
+ *   positive definite, bits 20-23 FP64 corrections (GSM_FP32_FP64FIX), bits
+ *   24-30 scalar iterations of the segment model that starts the line search.
+ *   The Norton law's step has its root on the predictor segment: it takes scalar
+ *   iterations (FP32) and one evaluation there, no Newton iteration of the full
+ *   system.
  */
 #ifndef GSM_GB300_H
 #define GSM_GB300_H

@@ -141,23 +141,27 @@ AD_HD float ray_seed(float L, float p, float inv_p, int& iters) {
 }
 
 struct RayRoot {
-  bool flows, bad;  // bad: the trial strain is not finite
+  bool flows;
+  bool bad;   // the trial strain is not finite, or its square is not
+  bool conv;  // no flow, or the last step met its tolerance
   int n_eval, n_model;
 };
 
 // The root in FP64: theta and t = 1 - theta, each to its own rounding.
 AD_HD RayRoot ray_root(const RayConst& c, double E2, bool active, double& theta, double& t) {
-  RayRoot r{false, false, 0, 0};
+  RayRoot r{false, false, true, 0, 0};
   theta = 0.0;
   t = 1.0;
   // E2 = 0 (a stress-free deviatoric state), NaN or out of range: no flow
   const int e2 = (int)((fpow::bits_of(E2) >> 52) & 0x7ff);
   r.bad = active && e2 > 1023 + 996;
+  r.conv = !r.bad;
   if (!active || e2 < 1023 - 996 || r.bad) return r;
   const float lgE = lg2_of(E2);
   const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
   if (!(u + 0.5f * lgE > c.lg_floor) || !(u > -1000.0f)) return r;
   r.flows = true;
+  r.conv = false;
   const float uf = floorf(u);
   double th = f64_of(ex2_approx(u - uf), (int)uf);
   for (int it = 0; it < 8; ++it) {
@@ -180,7 +184,10 @@ AD_HD RayRoot ray_root(const RayConst& c, double E2, bool active, double& theta,
     const double dth = th * step;
     theta = th + dth;
     t = s - dth;
-    if (!(fabsf(ef) > 8e-6f)) break;  // remainder below eta^3 / 10
+    if (!(fabsf(ef) > 8e-6f)) {  // remainder below eta^3 / 10
+      r.conv = ef == ef;
+      break;
+    }
     th = theta > 0.0 ? theta : 0.5 * th;
   }
   return r;
@@ -204,7 +211,7 @@ AD_HD df df_bits(double x, int k) {
 // range (the caller takes ray_root).
 AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool active, RayRoot& r, double& theta,
                        double& t) {
-  r = RayRoot{false, false, 0, 0};
+  r = RayRoot{false, false, true, 0, 0};
   theta = 0.0;
   t = 1.0;
   if (!active) return true;
@@ -262,8 +269,8 @@ AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool act
 }
 
 AD_HD unsigned ray_status(const RayRoot& r, bool correction) {
-  unsigned st = ST_CONVERGED | ((unsigned)(r.n_model & 0x7f) << ST_MODEL_SHIFT);
-  if (r.bad) st |= ST_NONFINITE;
+  unsigned st = r.conv ? ST_CONVERGED : r.bad ? ST_NONFINITE : ST_CAP;
+  st |= (unsigned)(r.n_model & 0x7f) << ST_MODEL_SHIFT;
   if (correction)
     st |= ((unsigned)r.n_eval << ST_NEWTON_SHIFT) | ((unsigned)(r.n_eval & 0xf) << ST_FIX_SHIFT);
   else
@@ -436,13 +443,15 @@ AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (
   for (int i = 0; i < 6; ++i) ss[i] = es[i] * inv_s;
   const float E2 = ss[0] * ss[0] + ss[1] * ss[1] + ss[2] * ss[2] +
                    0.5f * (ss[3] * ss[3] + ss[4] * ss[4] + ss[5] * ss[5]);  // in [0.5, 24)
-  RayRoot r{false, active && !(E2 < 1e30f), 0, 0};
+  const bool bad = active && !(E2 < 1e30f);
+  RayRoot r{false, bad, !bad, 0, 0};
   float theta = 0.0f, t = 1.0f;
   if (active && E2 > 0.0f && E2 < 1e30f) {
     const float lgE = lg2_approx(E2) + 2.0f * (float)k;
     const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
     if (u > -120.0f) {
       r.flows = true;
+      r.conv = false;
       float th = ex2_approx(u);
       for (int it = 0; it < 4; ++it) {
         ++r.n_eval;
@@ -465,7 +474,10 @@ AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (
         const float dth = th * (eta - eta * q * rcp_approx(1.0f + q));
         theta = th + dth;
         t = s - dth;
-        if (!(fabsf(eta) > 1e-3f)) break;
+        if (!(fabsf(eta) > 1e-3f)) {
+          r.conv = eta == eta;
+          break;
+        }
         th = theta > 0.0f ? theta : 0.5f * th;
       }
     }
