@@ -12,7 +12,8 @@
 // sweeps, a 5x5 factorisation).  With A = -d.psi_y(e_s, 0) = 2 mu (e_s:e_s)
 // and d.phi_v(theta d/h) = 2 mu (e_s:e_s) k(theta) the root solves
 //   k(theta) = 1 - theta,   k(theta) = c0 theta (E2 theta^2)^(a_phi - 1),  E2 = e_s:e_s,
-//   c0 = 2 a_phi c_phi / (3 mu h) (2 / (3 h^2))^(a_phi - 1)      (once per step),
+//   c0 = 2 a_phi c_phi / (3 mu h) (2 / (3 h^2))^(a_phi - 1)      (once per step;
+//   where that leaves the FP64 range, n < 0.1, on E2 scaled by a power of four),
 // and with t = 1 - theta
 //   w = theta d,   sigma = kappa tr(eps) 1 + 2 mu t e_s,
 //   C_t = kappa 1x1 + 2 mu t I_dev - 2 mu (1 - p) theta t / (p t + theta) n x n,
@@ -46,11 +47,12 @@ namespace gsm {
 // Constants of the scalar equation of one law and one step size.
 struct RayConst {
   double c0, am1, p, mu, kappa;
+  int sh;          // c0 belongs to 2^(2 sh) E2 (0 but where c0 of E2 itself is out of range)
   float am1f, pf, inv_pf, muf, kappaf;
   float lg_c0;     // log2 c0
   float c0m;       // c0 = c0m 2^c0e, c0m in [1, 2)
   int c0e;
-  float lg_floor;  // log2 of 1e-140 h: rates below 1e-140 of |d| / h are no flow
+  float lg_floor;  // log2 of 1e-140 h (2^sh): rates below 1e-140 of |d| / h are no flow
   df am1d, pd, c0d;  // am1, p and c0 2^-c0e as double-float pairs (the FP32-bulk correction)
 };
 
@@ -100,6 +102,13 @@ AD_HD RayConst make_ray(const LawParams<double>& p, double h) {
   r.mu = p.mu;
   r.kappa = p.lam + p.mu * (2.0 / 3.0);
   r.c0 = 2.0 * p.a_phi * p.c_phi / (3.0 * p.mu * h) * ::pow(2.0 / (3.0 * h * h), r.am1);
+  r.sh = 0;
+  if (p.L_ode > 0.0 && !(r.c0 > 1e-120 && r.c0 < 1e120)) {
+    // the same as C (X E2 theta^2)^(a_phi - 1) theta with C = sigma0 / (3 mu h edot0) and X = 2 / (3 h^2 edot0^2)
+    const double C = 1.0 / (p.L_ode * h), X = 0.5 * p.q_ode * C * C;
+    r.sh = (int)::rint(0.5 * ::log2(X));
+    r.c0 = C * ::pow(::ldexp(X, -2 * r.sh), r.am1);
+  }
   r.am1f = (float)r.am1;
   r.pf = (float)r.p;
   r.inv_pf = (float)(1.0 / r.p);
@@ -108,7 +117,7 @@ AD_HD RayConst make_ray(const LawParams<double>& p, double h) {
   r.lg_c0 = (float)::log2(r.c0);
   r.c0e = (int)((fpow::bits_of(r.c0) >> 52) & 0x7ff) - 1023;
   r.c0m = f32_of(r.c0, -r.c0e);
-  r.lg_floor = (float)::log2(1e-140 * h);
+  r.lg_floor = (float)(::log2(1e-140 * h) + r.sh);
   r.am1d = df_of(r.am1);
   r.pd = df_of(r.p);
   r.c0d = df_of(r.c0, -r.c0e);
@@ -153,10 +162,11 @@ AD_HD RayRoot ray_root(const RayConst& c, double E2, bool active, double& theta,
   theta = 0.0;
   t = 1.0;
   // E2 = 0 (a stress-free deviatoric state), NaN or out of range: no flow
-  const int e2 = (int)((fpow::bits_of(E2) >> 52) & 0x7ff);
-  r.bad = active && e2 > 1023 + 996;
+  const int e2 = (int)((fpow::bits_of(E2) >> 52) & 0x7ff), e2s = e2 + 2 * c.sh;
+  r.bad = active && (e2 > 1023 + 996 || e2s > 1023 + 996);
   r.conv = !r.bad;
-  if (!active || e2 < 1023 - 996 || r.bad) return r;
+  if (!active || e2 < 1023 - 996 || e2s < 1023 - 996 || r.bad) return r;
+  E2 = fpow::double_of(fpow::bits_of(E2) + ((uint64_t)(int64_t)(2 * c.sh) << 52));
   const float lgE = lg2_of(E2);
   const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
   if (!(u + 0.5f * lgE > c.lg_floor) || !(u > -1000.0f)) return r;
@@ -233,7 +243,7 @@ AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool act
   const df u2 = dfo::two_sum(n.hi, 0.5f * h.hi);
   const df E2 = dfo::fast_two_sum(u2.hi, dfo::add_rn(u2.lo, dfo::fma_rn(0.5f, h.lo, n.lo)));
   if (!(E2.hi > 0.25f && E2.hi < 64.0f)) return false;  // zero, non-finite or subnormal trial strain
-  const float lgE = lg2_approx(E2.hi) + 2.0f * (float)k;
+  const float lgE = lg2_approx(E2.hi) + 2.0f * (float)(k + c.sh);
   const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
   if (!(u > -40.0f)) return false;
   float th = ex2_approx(u);
@@ -244,7 +254,7 @@ AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool act
     const float t2 = dfo::mul_rn(tm, tm);
     const df x = E2 * df{t2, dfo::fma_rn(tm, tm, -t2)};
     df F;
-    if (!dpow::pow_scaled(x, 2 * (k + et), c.am1, c.am1d, c.c0d, c.c0e, F)) return false;
+    if (!dpow::pow_scaled(x, 2 * (k + c.sh + et), c.am1, c.am1d, c.c0d, c.c0e, F)) return false;
     const df kk = F * th;
     const df s = dfo::two_sum(1.0f, -th);
     const df R = s - kk;
@@ -391,14 +401,14 @@ AD_HD void ray_flow_apply(double mu, double p, double theta, double t, double E2
   for (int a = 0; a < 5; ++a) out[a] = f * (Mb[a] + w * Md[a]);
 }
 
-// FP32 power (2^e m)^a with lgm = log2 m: the product a e is split into its
-// integer part and an exact remainder, so the result carries ~2^-23, not
-// 2^-23 of the exponent.  Returns r with the power = 2^n r.
+// FP32 power (2^e m)^a with lgm = log2 m: the integer nearest the exponent is
+// split off and the product a e kept with its remainder, so the result carries
+// ~2^-23, not 2^-23 of the exponent.  Returns r with the power = 2^n r.
 AD_HD float ray_pow(float a, int e, float lgm, int& n) {
   const float ef = (float)e;
   const float yh = a * ef;
   const float yl = fmaf(a, ef, -yh);
-  const float ni = rintf(yh);
+  const float ni = rintf(fmaf(a, lgm, yh));
   n = (int)ni;
   return ex2_approx((yh - ni) + fmaf(a, lgm, yl));
 }
@@ -447,7 +457,7 @@ AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (
   RayRoot r{false, bad, !bad, 0, 0};
   float theta = 0.0f, t = 1.0f;
   if (active && E2 > 0.0f && E2 < 1e30f) {
-    const float lgE = lg2_approx(E2) + 2.0f * (float)k;
+    const float lgE = lg2_approx(E2) + 2.0f * (float)(k + c.sh);
     const float u = ray_seed(c.lg_c0 + c.am1f * lgE, c.pf, c.inv_pf, r.n_model);
     if (u > -120.0f) {
       r.flows = true;
@@ -462,7 +472,7 @@ AD_HD unsigned voxel_ray(const RayConst& c, const float (&eps)[6], const float (
         const float x = E2 * tm * tm;
         const int ex = ilog2_pos(x);
         int n;
-        const float pw = ray_pow(c.am1f, ex + 2 * (k + et), lg2_approx(x * exp2i(-ex, 0.0f)), n);
+        const float pw = ray_pow(c.am1f, ex + 2 * (k + c.sh + et), lg2_approx(x * exp2i(-ex, 0.0f)), n);
         n += c.c0e;
         n = n > 240 ? 240 : (n < -240 ? -240 : n);
         const int n1 = n / 2;
