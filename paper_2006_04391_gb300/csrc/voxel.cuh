@@ -2,7 +2,7 @@
 // consistent tangent.  Used by the batch kernel (gsm_update) and by the
 // material kernel of the basic scheme.
 //
-//   MODE_FP64       every step in FP64.
+//   MODE_FP64       every step in FP64 (the scalar equation: from an FP32 start).
 //   MODE_FP32_FIX   FP32 line search and Newton (the bulk of the work), then
 //                   FP64 Newton corrections: FP64 residual, the FP32 Newton
 //                   matrix of the last FP32 iteration, until the correction is
@@ -13,7 +13,10 @@
 //
 // A proportional law (Law::kRay) takes the scalar equation of ray.cuh in all
 // three modes; what follows below is the general path, for a law whose
-// implicit-Euler step needs the full Newton system.
+// implicit-Euler step needs the full Newton system.  No law the library ships
+// is one (the Michel-Suquet law is integrated by the ODE updates only), so no
+// kernel instantiates it: host tests hold it to the oracle and the scalar
+// equation to it.
 #pragma once
 
 #include "ray.cuh"
