@@ -39,6 +39,7 @@ constexpr int kOdeBlock = 128;
 // half an attempt; waiting costs idle lanes.  Measured on 200 k voxels, n = 5:
 // 3645 us with 1, 3502 with 4, 3686 with 8, 4108 with 12.
 constexpr int kRefill = 4;
+constexpr int kOdeGroup = 8;  // voxels: whole 32-byte sectors of every component
 
 // Per-lane scheduling (without the tangent): a lane starts its next voxel when
 // its current one has finished its substeps; the warp runs while any lane has
@@ -99,16 +100,20 @@ __global__ void __launch_bounds__(kOdeBlock) ode23_kernel(int64_t n, int64_t ld,
     }
     return;
   }
-  // a block owns a contiguous range of voxels; its lanes take the next one of it
-  // from a shared counter, so they finish together whatever their substep counts
-  // (200 k voxels: 3502 -> 3174 us against a fixed stride per lane)
-  const int64_t per = (n + gridDim.x - 1) / gridDim.x, first = (int64_t)blockIdx.x * per;
-  const int64_t last = first + per < n ? first + per : n;
+  // a block owns every gridDim-th group of kOdeGroup voxels; its lanes take the next
+  // one of them from a shared counter, so they finish together whatever their
+  // substep counts (200 k voxels: 3502 -> 3177 us against a fixed stride per lane).
+  // Groups and not one range: where the flow is confined to a part of the field,
+  // the blocks of that part would work alone (1 M voxels, 2 % of them flowing,
+  // ode23 5772 -> 1010 us, ode12 18042 -> 2392).
   __shared__ unsigned long long taken;
   if (threadIdx.x == 0) taken = blockDim.x;
   __syncthreads();
-  i = first + threadIdx.x;
-  bool have = i < last;
+  auto voxel = [&](int64_t k) {
+    return ((k / kOdeGroup) * gridDim.x + blockIdx.x) * kOdeGroup + k % kOdeGroup;
+  };
+  i = voxel(threadIdx.x);
+  bool have = i < n;
   if (have) start(i);
   for (;;) {
     const bool busy = have && !v.done;
@@ -125,8 +130,8 @@ __global__ void __launch_bounds__(kOdeBlock) ode23_kernel(int64_t n, int64_t ld,
 #pragma unroll
         for (int c = 0; c < NZ; ++c) z[c * ld + i] = zo[c];
         if (status) status[i] = (int32_t)st;
-        i = first + (int64_t)atomicAdd(&taken, 1ull);
-        have = i < last;
+        i = voxel((int64_t)atomicAdd(&taken, 1ull));
+        have = i < n;
         if (have) start(i);
       }
     }
