@@ -128,7 +128,9 @@ int gsm_update(gsm_handle h, int64_t n_vox, const void* eps, const void* z_n, in
 /*
  * gsm_update_host -- gsm_update for arrays that live in page-locked host memory.
  * chunk = 0: the kernel reads and writes them directly over the host link (as
- * gsm_update does), or, where the device cannot address them, in chunks of 2^17.
+ * gsm_update does); in chunks of 2^18 or 2^19 where rows off 32-byte boundaries
+ * (an odd ld) are so long that the copies are the faster way, and of 2^17 where
+ * the device cannot address the arrays.
  * chunk > 0: streamed through the device in chunks of `chunk` voxels: the
  * host->device copies of chunk i+1 and the device->host copies of chunk i-1
  * (two internal streams, the copy engines of both directions of the host link)

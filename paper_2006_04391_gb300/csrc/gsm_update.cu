@@ -12,6 +12,7 @@
 #include <mutex>
 
 #include <algorithm>
+#include <limits>
 
 #include "common.cuh"
 #include "voxel.cuh"
@@ -190,6 +191,49 @@ bool device_address(const void* p, const void** out) {
   }
 }
 
+// Device addresses of the arrays of an update; ok: the device reaches them all.
+struct Mapped {
+  const void* in[2];
+  void* out[4];
+  bool ok;
+};
+Mapped map_arrays(const void* eps, const void* z_n, void* sigma, void* z, void* tangent, int32_t* status) {
+  Mapped a{{eps, z_n}, {sigma, z, tangent, status}, true};
+  for (auto& p : a.in) a.ok = device_address(p, &p) && a.ok;
+  for (auto& p : a.out) {
+    const void* q = p;
+    a.ok = device_address(q, &q) && a.ok;
+    p = const_cast<void*>(q);
+  }
+  return a;
+}
+
+// Whether gsm_update_host without a chunk size stages its rows: they start off
+// 32-byte boundaries and are long.  us, rows at an odd ld, direct / staged (2^18,
+// from 2^21 voxels 2^19):
+//   FP32             2^20  505 /  554   2^21  965 /  987   2^22 1983 / 1832   2^23  4214 /  3431
+//   FP32 + tangent   2^18  319 /  345   2^19  616 /  578   2^20 1209 / 1043   2^23  9908 /  7125
+//   FP64 (+ bulk)    2^21 1606 / 1857   2^23 6495 / 6533
+//   FP64 + tangent   2^20 1960 / 1945   2^21 3861 / 3818   2^22 7747 / 7182   2^23 15386 / 13910
+// (at 32-byte boundaries direct is the faster one at every size, 2^21 FP32: 850 /
+// 953).  Never under stream capture, where the copies' streams would be created.
+bool stage_rows(int precision, int64_t n, int64_t ld, const void* eps, const void* z_n, const void* sigma,
+                const void* z, const void* tangent, cudaStream_t s) {
+  const bool f32 = precision == GSM_FP32;
+  const int64_t least = f32 ? (tangent ? (int64_t)1 << 19 : (int64_t)1 << 22)
+                            : (tangent ? (int64_t)1 << 21 : std::numeric_limits<int64_t>::max());
+  if (n < least || (z && !z_n)) return false;
+  uintptr_t at = (uintptr_t)ld * (f32 ? sizeof(float) : sizeof(double));
+  for (const void* p : {eps, z_n, sigma, z, tangent}) at |= reinterpret_cast<uintptr_t>(p);
+  if (at % 32 == 0) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
 int validate_material(int psi_kind, int phi_kind, const double* prm, int n_params, int precision) {
   if (!prm) return GSM_EINVAL;
   if (precision < GSM_FP64 || precision > GSM_FP32) return GSM_EINVAL;
@@ -250,17 +294,10 @@ int gsm_update(gsm_handle h, int64_t n_vox, const void* eps, const void* z_n, in
   // every array may be device memory or page-locked host memory (read and
   // written by the kernel over the host link); unregistered host memory is
   // refused rather than faulted on
-  const void* in[2] = {eps, z_n};
-  void* out[4] = {sigma, z, tangent, status};
-  for (auto& p : in)
-    if (!device_address(p, &p)) return GSM_EINVAL;
-  for (auto& p : out) {
-    const void* q = p;
-    if (!device_address(q, &q)) return GSM_EINVAL;
-    p = const_cast<void*>(q);
-  }
-  return material_update(m, n_vox, in[0], in[1], ld, step_h, out[0], out[1], out[2], static_cast<int32_t*>(out[3]),
-                         static_cast<cudaStream_t>(stream));
+  const Mapped a = map_arrays(eps, z_n, sigma, z, tangent, status);
+  if (!a.ok) return GSM_EINVAL;
+  return material_update(m, n_vox, a.in[0], a.in[1], ld, step_h, a.out[0], a.out[1], a.out[2],
+                         static_cast<int32_t*>(a.out[3]), static_cast<cudaStream_t>(stream));
 }
 
 // Chunked host <-> device streaming of gsm_update: three slots of device
@@ -293,21 +330,17 @@ int gsm_update_host(gsm_handle h, int64_t n_vox, const void* eps, const void* z_
   // voxels, 384 MB) 1630 us against 2270 us for the best staged chunk (2^17) and
   // 3340 us for 2^20, and 31 against 300 us at 10 k voxels: no copies, no staging
   // buffers, and both directions of the link busy from the first warp on.
-  if (chunk == 0) {
-    const void* in[2] = {eps, z_n};
-    void* out[4] = {sigma, z, tangent, status};
-    bool mapped = true;
-    for (auto& p : in) mapped = mapped && device_address(p, &p);
-    for (auto& p : out) {
-      const void* q = p;
-      mapped = mapped && device_address(q, &q);
-      p = const_cast<void*>(q);
-    }
-    if (mapped)
-      return material_update(m, n_vox, in[0], in[1], ld, step_h, out[0], out[1], out[2], static_cast<int32_t*>(out[3]),
-                             static_cast<cudaStream_t>(stream));
-  }
-  const int64_t C = std::min<int64_t>(chunk > 0 ? chunk : (int64_t)1 << 17, n_vox);
+  // Not where the rows are long and start off the link's 32-byte sectors (an odd
+  // ld): a warp's 32 values then straddle one more sector in every row, which costs
+  // FP32 rows, and the many written rows of a tangent, more than the copies do.
+  const Mapped io = chunk == 0 ? map_arrays(eps, z_n, sigma, z, tangent, status) : Mapped{};
+  const bool stage = chunk == 0 && stage_rows(m.precision, n_vox, ld, eps, z_n, sigma, z, tangent,
+                                              static_cast<cudaStream_t>(stream));
+  if (chunk == 0 && io.ok && !stage)
+    return material_update(m, n_vox, io.in[0], io.in[1], ld, step_h, io.out[0], io.out[1], io.out[2],
+                           static_cast<int32_t*>(io.out[3]), static_cast<cudaStream_t>(stream));
+  const int64_t C =
+      std::min<int64_t>(chunk > 0 ? chunk : !stage ? (int64_t)1 << 17 : (int64_t)1 << (n_vox >> 21 ? 19 : 18), n_vox);
   const size_t es = m.precision == GSM_FP32 ? sizeof(float) : sizeof(double);
   const bool use_z = z_n && z;  // (the elastic law copies z_n into z when both are given)
   // per slot: eps, z_n, sigma, z [6][C]; tangent [21][C]; status [C]
@@ -318,6 +351,9 @@ int gsm_update_host(gsm_handle h, int64_t n_vox, const void* eps, const void* z_
   char* buf = nullptr;
   if (cudaMallocAsync((void**)&buf, kSlots * slot, cs) != cudaSuccess) {
     cudaGetLastError();
+    if (stage && io.ok)
+      return material_update(m, n_vox, io.in[0], io.in[1], ld, step_h, io.out[0], io.out[1], io.out[2],
+                             static_cast<int32_t*>(io.out[3]), cs);
     return GSM_ENOMEM;
   }
   cudaStream_t in_s = nullptr, out_s = nullptr;
