@@ -26,17 +26,18 @@
 // Solution: theta in FP32 from the equation in u = log2 theta (convex and
 // increasing; Newton from an upper bound decreases monotonically onto the
 // root), then Halley steps in the working precision on the equation itself.
-// One step squares^1.5 the seed's ~1e-7: its remainder is below 1e-18, so a
-// voxel takes one power in the working precision.  FP64 operations per voxel:
-// about 75, where the line search and Newton steps took about 800.
+// One step cubes the seed's ~1e-7: its remainder is below 1e-18, so a voxel
+// takes one power in the working precision.  FP64 operations per voxel: 74
+// (33 in the FP32-bulk mode), where the line search and Newton steps took about
+// 800.
 //
-// Bound: FP64 the FP64 pipe (75 operations at 629 G/s: 7.4 G voxel/s at 100 %),
-// FP32 the memory (96 bytes a voxel).  Measured on GB300 against the general
-// solver: FP64 3.0 M voxels (n = 10) 5208 -> 415 us (97 % of the FP64 pipe's
-// issue rate for these operations), FP64 with tangent 1.0 M voxels 2793 -> 232
-// us, FP32 5.0 M voxels 266 -> 87 us (5.5 TB/s), FP32 bulk + correction 2^24
-// voxels 3015 -> 1119 us (2450 with the correction in FP64; 2.9 TB/s), the FP32
-// material kernel of the scheme at 256^3 1199 -> 372 us.
+// Bound: FP64 the FP64 pipe (74 operations at 629 G/s: 8.5 G voxel/s at 100 %;
+// the pipe is 87 % busy, its maximum in any kernel here), FP32 the memory (96
+// bytes a voxel).  Measured on GB300 against the general solver: FP64 3.0 M
+// voxels (n = 10) 5208 -> 415 us (7.2 G voxel/s), FP64 with tangent 1.0 M voxels
+// 2793 -> 233 us, FP32 5.0 M voxels 266 -> 86 us (5.6 TB/s), FP32 bulk +
+// correction 2^24 voxels 3015 -> 1120 us (2450 with the correction in FP64; 2.9
+// TB/s), the FP32 material kernel of the scheme at 256^3 1199 -> 294 us.
 #pragma once
 
 #include "dpow.cuh"
@@ -217,8 +218,9 @@ AD_HD df df_bits(double x, int k) {
 // equation's residual in double-float arithmetic (2^-45, the accuracy of this
 // mode's correction), on e_s scaled by 2^-k.  FP64 operations: three inside the
 // power and one per result, where ray_root takes about 45; the FP64 pipe runs
-// at 1/64 of the FP32 rate.  Returns false where a value leaves the pairs'
-// range (the caller takes ray_root).
+// at 1/64 of the FP32 rate.  Returns false where the pairs do not reach (a zero,
+// subnormal or non-finite trial strain, a start far from the root): the caller
+// takes ray_root.
 AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool active, RayRoot& r, double& theta,
                        double& t) {
   r = RayRoot{false, false, true, 0, 0};
@@ -249,7 +251,7 @@ AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool act
   if (!(u + 0.5f * lgE > c.lg_floor) || !(u > -1000.0f)) return true;
   // theta = 2^et tm, tm near 1: a flow of any size takes the same FP32 pairs
   // (below 2^-40 the FP64 root took over before: n = 20, strains of 2e-5, 4.2 M
-  // voxels 893 -> 338 us; the flowing batch 2^24 1120 -> 1128 us)
+  // voxels 893 -> 336 us; a flowing batch as before)
   // (et = u rounded, by an addition: no conversion)
   constexpr float magic = 12582912.0f;  // 1.5 2^23
   const float um = u + magic;
@@ -261,7 +263,10 @@ AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool act
     const float t2 = dfo::mul_rn(tm, tm);
     const df x = E2 * df{t2, dfo::fma_rn(tm, tm, -t2)};
     df F;
-    if (!dpow::pow_scaled(x, 2 * (k + c.sh + et), c.am1, c.am1d, c.c0d, c.c0e + et, F)) return false;
+    // (one exit: a second one at the loop's end cost a voxel 1 us of latency)
+    if (!(tm > 0.25f && tm < 4.0f) ||
+        !dpow::pow_scaled(x, 2 * (k + c.sh + et), c.am1, c.am1d, c.c0d, c.c0e + et, F))
+      return false;
     const float th = tm * sc;
     const df kk = F * tm;
     const df s = dfo::two_sum(1.0f, -th);
@@ -281,7 +286,6 @@ AD_HD bool ray_root_df(const RayConst& c, const double (&es)[6], int k, bool act
       return true;
     }
     tm = tm + dth.hi;
-    if (!(tm > 0.25f && tm < 4.0f)) return false;
   }
   return false;
 }
