@@ -77,10 +77,11 @@ OPS_FIX_EXTRA = 5.0
 OPS_FP64_BASE = 32.05
 OPS_FP64_LINE = 42.0
 BYTES_PER_VOXEL_FP64 = 4 * 6 * 8          # eps, z_n in; sigma, z out
-# DRAM bytes of one full-size FP32-bulk launch (ncu dram__bytes_read.sum +
-# dram__bytes_write.sum, one capture of launch 6 of this workload: the
-# inputs are read once, less what the 129 MB L2 still holds)
-TRAFFIC_FP32FIX = 1476579840 + 1630033408
+# DRAM bytes of one full-size FP32-bulk launch of this kernel (ncu
+# dram__bytes_read.sum + dram__bytes_write.sum, one capture of this workload,
+# profiles/norton_kernel_fp32fix_traffic_2p24.md: the inputs are read once, less
+# what the 129 MB L2 still holds); a constant, not measured in the run
+TRAFFIC_FP32FIX = 1476515328 + 1642326016
 
 
 # The paper's own figures for this path (context, other hardware and workload:

@@ -356,7 +356,7 @@ typedef struct ms_tape* ms_tape_handle;
 
 /* ms_run_taped -- ms_run from a fresh state (no resume) that keeps the
  * checkpoints (eps_k, z_{k-1}) of every step on the device (2 * 6 * N^3
- * doubles per step) plus adjoint work arrays (53 * N^3 doubles).  The tape
+ * doubles per step) plus adjoint work arrays (59 * N^3 doubles).  The tape
  * refers to the context, which must outlive it.  Prescribed macroscopic
  * strains and the implicit-Euler update only (stress_mask = 0, integrator =
  * 0; GSM_ENOTSUP otherwise); the reference medium may be fixed or per step

@@ -248,8 +248,10 @@ def gsm_update(mat, eps, z_n, h, sigma, z, tangent=None, status=None, stream=Non
 
 def gsm_update_host(mat, eps, z_n, h, sigma, z, tangent=None, status=None, chunk=0, stream=None, n_vox=None):
     """gsm_update on pinned CPU tensors (``[6, ld]``, tangent ``[21, ld]``, status
-    ``[ld]``), streamed through the device in chunks with copies overlapping the
-    updates; asynchronous on ``stream``."""
+    ``[ld]``); asynchronous on ``stream``.  chunk = 0: the kernel works on the host
+    memory itself, or the library chooses a chunk (long rows off 32-byte
+    boundaries); chunk > 0: streamed through the device in chunks with copies
+    overlapping the updates."""
     lib = load()
     ld = eps.shape[1]
     n = ld if n_vox is None else int(n_vox)

@@ -11,13 +11,16 @@
 // Bound: FP32 the memory, FP64 the FP64 pipe (a 256-point line takes about 6000
 // operations in two radix-16 stages).  Measured on GB300 against cuFFT with the
 // separate Green kernel, one iteration's transforms and update: FP32 256^3
-// 1.21 -> 0.97 ms, FP64 256^3 22.6 -> 15.0 ms; with the smaller chunks of the
-// reductions the 16^3 FP64 iteration 400 -> 45 us.
+// 1.21 -> 1.00 ms, FP64 256^3 22.6 -> 14.9 ms; with the smaller chunks of the
+// reductions the 16^3 FP64 iteration 400 -> 44 us.
 //
 // Layout (as cuFFT's): real [6][N][N][N], spectrum [6][N][N][Nh], Nh = N/2 + 1,
 // unnormalised both ways; the forward passes give twice the spectrum (the
 // separation of the two lines of a z pair leaves out its factor 1/2, an exact
-// scaling that the constants of what follows take).  N = R1 R2 with R1, R2 <= 16, N even.
+// scaling that the constants of what follows take).  N = R1 R2, both among the
+// radices below (at most 16), N even: the sizes listed in fft_f32*.cu and
+// fft_f64*.cu.  Other sizes (factors of 7, N > 256, even sizes not listed) take
+// cuFFT.
 //
 // One line of N = R1 R2 points by two register stages and one exchange
 // through shared memory (n = n1 R2 + n2, k = k1 + R1 k2):
@@ -224,7 +227,7 @@ template <class T, int N> struct Shape {
   // blocks an SM, whose phases then overlap (FP32 128^3 66 -> 45 us, FP64 256^3
   // 5.75 -> 5.57 ms against all six at once); where a block takes more than
   // half an SM's shared memory anyway (FP32, N > 200) all six at once are
-  // faster (256^3: 416 against 474 us).
+  // faster (256^3: 445 against 503 us).
   static constexpr int GW = (sizeof(T) == 4 ? 8 : 4), CG = (sizeof(T) == 4 && N > 200) || 6 * TPL * GW <= 256 ? 6 : 2;
   static constexpr int GL = CG * TPL * GW;            // threads that hold lines
   static constexpr int GT = (GL + 31) / 32 * 32;       // whole warps (the block sum)

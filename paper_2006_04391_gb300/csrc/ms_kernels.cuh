@@ -400,8 +400,8 @@ __device__ __forceinline__ int owner(const int64_t* starts, int n, int64_t c) {
 }
 
 // Batched material evaluation: all jobs of the launch, chunk by chunk.
-// (FP32: 40 registers, twelve blocks an SM, 24 bytes spilled; the kernel waits on
-// loads: 256^3 385 us at nine blocks, 306 at ten, 300 at twelve, 346 at sixteen)
+// (FP32: 40 registers, twelve blocks an SM, 20 bytes spilled; the kernel waits on
+// loads: 256^3 385 us at nine blocks, 306 at ten, 294 at twelve, 346 at sixteen)
 template <class T, int MODE>
 __global__ void __launch_bounds__(kMatBlock, MODE == MODE_FP32 ? 12 : 1) ms_material_batch_kernel(const JobView* __restrict__ views, int n_jobs,
                                                                       int64_t total_chunks) {
