@@ -64,15 +64,14 @@ def test_long_odd_rows_are_not_slower_than_staged(gsm):
     import torch
     mat, _, host = arrays(gsm, (1 << 22) + 9, 2, True)
 
-    def best(**kw):
-        times = []
-        for _ in range(5):
+    times = {0: [], 1 << 19: []}
+    for _ in range(10):  # in turn: the link's rate drifts by some percent
+        for chunk, out in times.items():
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record()
-            call(gsm.gsm_update_host, mat, host, **kw)
+            call(gsm.gsm_update_host, mat, host, chunk=chunk)
             b.record()
             torch.cuda.synchronize()
-            times.append(a.elapsed_time(b))
-        return min(times[1:])
-
-    assert best() < 1.15 * best(chunk=1 << 19)  # (1.3 times by the kernel on the host memory)
+            out.append(a.elapsed_time(b))
+    direct, staged = (min(t[1:]) for t in times.values())
+    assert direct < 1.15 * staged  # (1.3 times by the kernel on the host memory)
